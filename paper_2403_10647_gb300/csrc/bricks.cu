@@ -1,0 +1,858 @@
+// Brick builds (sm_103a): RadixSort, RunLengthEncode, NonEmptyCells and
+// ExclusiveSum of Algorithm 1 over bricks of cells instead of single cells.
+//
+// A triangle's pairs fill a box of cells, so the sort need not carry them one
+// by one.  The grid is cut into bricks (8 x 8 x 8 cells); the sorted entries are
+// (brick, object) with the object's box inside the brick packed into the spare
+// key and value bits (BrickGen): 1.2 to 1.6 entries per triangle on the
+// scenes of scenes/, against 3 to 140 pairs.  The stable radix passes leave
+// every brick's entries in ascending object order, and the pairs first appear
+// in device memory as the final refs.
+//
+//   split   work items: a brick's entries, at most BRICK_CHUNK each.
+//   count   objects per cell.
+//   scan    exclusive sums of the counts: G (localized per mesh in a batch).
+//   fill    refs: every cell's objects in ascending order at G[cell].
+//
+// count and fill find the objects of a cell by bit masks.  32 entries at a
+// time, a warp turns the boxes into 32 rows of feature bits (columns x, rows
+// y, layers z that the box covers) and transposes them, so that lane f holds
+// which of the 32 entries cover feature f; the entries covering cell (x, y, z)
+// are then X[x] & Y[y] & Z[z].  No atomics, no per-pair search, and ascending
+// bits are ascending objects.
+#include <atomic>
+#include <cstdint>
+
+#include "device.cuh"
+#include "kernels.h"
+
+namespace gg {
+
+namespace {
+
+constexpr unsigned FULL = 0xFFFFFFFFu;
+constexpr unsigned NO_SLOT = 0xFFFFFFFFu;
+constexpr int GROUPS = BRICK_CELLS / 32;   // groups of 32 cells, in cell order
+
+// Decoded BrickItem::dims.
+struct Dims {
+    unsigned nx, ny, nz;   // cells inside the grid per axis
+    unsigned lx, ly, lz;
+};
+
+__device__ __forceinline__ Dims decode(unsigned d)
+{
+    return Dims{(d & 31u) + 1u, ((d >> 5) & 31u) + 1u, ((d >> 10) & 31u) + 1u, (d >> 15) & 7u, (d >> 18) & 7u,
+                (d >> 21) & 7u};
+}
+
+__device__ __forceinline__ BrickItem load_item(const BrickItem *p)
+{
+    const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p)), b = __ldg(reinterpret_cast<const uint4 *>(p) + 1);
+    return BrickItem{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+}
+
+// Bits a .. b (inclusive) set.
+__device__ __forceinline__ unsigned bit_run(unsigned a, unsigned b) { return (2u << b) - (1u << a); }
+
+// Feature bits of an entry's box: columns at bit 0, rows at 2^lx, layers at
+// 2^lx + 2^ly.
+__device__ __forceinline__ unsigned feature_row(unsigned info, const Dims &d)
+{
+    const unsigned l0 = info & (BRICK_CELLS - 1u), l1 = (info >> BRICK_CELLS_LOG) & (BRICK_CELLS - 1u);
+    const unsigned mx = (1u << d.lx) - 1u, my = (1u << d.ly) - 1u, mz = (1u << d.lz) - 1u;
+    const unsigned lxy = d.lx + d.ly;
+    const unsigned X = bit_run(l0 & mx, l1 & mx);
+    const unsigned Y = bit_run((l0 >> d.lx) & my, (l1 >> d.lx) & my);
+    const unsigned Z = bit_run((l0 >> lxy) & mz, (l1 >> lxy) & mz);
+    return X | (Y << (1u << d.lx)) | (Z << ((1u << d.lx) + (1u << d.ly)));
+}
+
+// 32 x 32 bit transpose across the warp: bit j of lane i moves to bit i of
+// lane j.
+__device__ __forceinline__ unsigned transpose32(unsigned x)
+{
+    const unsigned lane = threadIdx.x & 31u;
+    unsigned m = 0x0000FFFFu;
+#pragma unroll
+    for (unsigned j = 16u; j; j >>= 1, m ^= m << j) {
+        const unsigned y = __shfl_xor_sync(FULL, x, j);
+        x = (lane & j) ? (x & ~m) | ((y & ~m) >> j) : (x & m) | ((y & m) << j);
+    }
+    return x;
+}
+
+// Entry e + k of an item (n entries left from e) in lane 31 - k, so that in a
+// transposed mask counting leading zeros walks the entries in ascending order.
+struct Entry {
+    unsigned key, val;
+    bool ok;
+};
+
+__device__ __forceinline__ Entry load_entry(const BrickArgs &a, unsigned e, unsigned n)
+{
+    const unsigned k = 31u - (threadIdx.x & 31u);
+    Entry r{0u, 0u, k < n};
+    if (r.ok) {
+        r.key = __ldg(a.keys + e + k);
+        r.val = __ldg(a.vals + e + k);
+    }
+    return r;
+}
+
+// The packed box, and the object.
+__device__ __forceinline__ unsigned entry_info(const BrickArgs &a, const Entry &r)
+{
+    return (r.key >> a.kb) | ((r.val >> a.ob) << brick_key_info_bits(a.kb));
+}
+
+__device__ __forceinline__ unsigned entry_obj(const BrickArgs &a, const Entry &r) { return r.val & ((1u << a.ob) - 1u); }
+
+// Mesh of a brick (the last m with brick_base[m] <= b; every mesh has bricks).
+__device__ __forceinline__ int mesh_of_brick(const MeshTab &mt, unsigned b)
+{
+    int lo = 0, hi = mt.nm - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (__ldg(&mt.md[mid].brick_base) <= b)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    return lo;
+}
+
+// First entry of brick b (b <= nbricks): the number of keys of bricks below b.
+__device__ __forceinline__ unsigned brick_start(const BrickArgs &a, unsigned b)
+{
+    if (b >= a.nbricks) return a.count;
+    const unsigned mask = (1u << a.kb) - 1u;
+    unsigned lo = 0, hi = a.count;
+    while (lo < hi) {
+        const unsigned mid = lo + ((hi - lo) >> 1);
+        if ((__ldg(a.keys + mid) & mask) < b)
+            lo = mid + 1u;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// split: bricks -> work items
+// ---------------------------------------------------------------------------
+
+// One thread per brick: its first entry by binary search, its items appended to
+// the list.  Empty bricks go to the other end of the list: only the count
+// visits them, to write their zeros.
+__global__ void __launch_bounds__(256) brick_split_kernel(BrickArgs a)
+{
+    __shared__ unsigned s_start[257];
+    __shared__ unsigned s_tmp[8];
+    __shared__ unsigned s_base, s_ebase;
+    const unsigned tid = threadIdx.x, b0 = blockIdx.x * 256u, b = b0 + tid;
+    if (b <= a.nbricks) s_start[tid] = brick_start(a, b);
+    if (tid == 255u && b + 1u <= a.nbricks) s_start[256] = brick_start(a, b + 1u);
+    __syncthreads();
+    const bool ok = b < a.nbricks;
+    BrickItem it{};
+    unsigned m = 0u, k = 0u;
+    if (ok) {
+        it.first = s_start[tid];
+        m = s_start[tid + 1] - it.first;
+        k = (m + BRICK_CHUNK - 1u) / BRICK_CHUNK;
+        unsigned shape = a.shape, nbx = a.nbx, nby = a.nby, lb = b;
+        int r[3] = {a.res[0], a.res[1], a.res[2]};
+        unsigned long long c0 = 0ull;
+        if (a.mt.md) {
+            const int q = mesh_of_brick(a.mt, b);
+            const MeshDesc &md = a.mt.md[q];
+            shape = md.shape;
+            nbx = md.nbx;
+            nby = md.nby;
+            lb = b - md.brick_base;
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) r[ax] = md.res[ax];
+            c0 = (unsigned long long)__ldg(a.cells_off + q);
+            it.base = __ldg(a.pair_base + q);
+        }
+        const unsigned lx = shape & 15u, ly = (shape >> 4) & 15u, lz = (shape >> 8) & 15u;
+        const unsigned bz = lb / (nbx * nby), rem = lb - bz * nbx * nby, by = rem / nbx, bx = rem - by * nbx;
+        const unsigned x0 = bx << lx, y0 = by << ly, z0 = bz << lz;
+        it.rx = (unsigned)r[0];
+        it.rxy = (unsigned)r[0] * (unsigned)r[1];
+        it.cell0 = (unsigned)(c0 + x0 + (unsigned long long)it.rx * (y0 + (unsigned long long)r[1] * z0));
+        const unsigned ex = min(1u << lx, (unsigned)r[0] - x0) - 1u, ey = min(1u << ly, (unsigned)r[1] - y0) - 1u,
+                       ez = min(1u << lz, (unsigned)r[2] - z0) - 1u;
+        it.dims = ex | (ey << 5) | (ez << 10) | (lx << 15) | (ly << 18) | (lz << 21);
+    }
+    unsigned total, etotal;
+    const unsigned ex = block_excl_sum<256>(k, s_tmp, &total);
+    const unsigned eex = block_excl_sum<256>(ok && m == 0u ? 1u : 0u, s_tmp, &etotal);
+    if (tid == 0u) {
+        s_base = total ? atomicAdd(&a.ctl->tickets[3], total) : 0u;
+        s_ebase = etotal ? atomicAdd(&a.ctl->tickets[6], etotal) : 0u;
+    }
+    __syncthreads();
+    if (ok && m == 0u) {
+        const unsigned p = s_ebase + eex;
+        it.count = 0u;
+        it.slot = NO_SLOT;
+        if (p < a.max_items)
+            a.items[a.max_items - 1u - p] = it;
+        else
+            atomicOr(&a.ctl->err, ERR_RANGE);
+    }
+    if (k) {
+        unsigned slot = NO_SLOT;
+        if (k > 1u) {
+            slot = atomicAdd(&a.ctl->tickets[4], k);
+            if (slot + k <= a.max_slots)
+                a.arrive[slot] = 0u;
+        }
+        const unsigned p = s_base + ex;
+        // never beyond: the host sizes both lists for every split of `count` entries
+        if (p + k > a.max_items || (k > 1u && slot + k > a.max_slots)) {
+            atomicOr(&a.ctl->err, ERR_RANGE);
+        } else {
+            const unsigned first = it.first;
+            for (unsigned j = 0; j < k; ++j) {
+                it.first = first + j * BRICK_CHUNK;
+                it.count = min((unsigned)BRICK_CHUNK, m - j * BRICK_CHUNK);
+                it.slot = k > 1u ? slot + j : NO_SLOT;
+                if (k > 1u) a.slot_meta[slot + j] = make_uint2(slot, k);
+                a.items[p + j] = it;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// count: objects per cell
+// ---------------------------------------------------------------------------
+
+constexpr int COUNT_WARPS = 4;
+
+// Adds an item's entries to cnt: lane l of group g counts cell 32 g + l.  The
+// next word's entries are loaded while one is counted.
+__device__ __forceinline__ void count_words(const BrickArgs &a, const BrickItem &it, const Dims &d,
+                                            unsigned (&cnt)[GROUPS])
+{
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned fy = 1u << d.lx, fz = fy + (1u << d.ly);
+    const bool cube = d.lx == 3u && d.ly == 3u && d.lz == 3u;
+    const int ngroups = max(1, 1 << (d.lx + d.ly + d.lz) >> 5);
+    Entry next = load_entry(a, it.first, it.count);
+    for (unsigned e = 0; e < it.count; e += 32u) {
+        const Entry cur = next;
+        const unsigned en = e + 32u;
+        next = load_entry(a, it.first + en, en < it.count ? it.count - en : 0u);
+        const unsigned f = transpose32(cur.ok ? feature_row(entry_info(a, cur), d) : 0u);
+        if (cube) {   // cell 32 g + l is (l % 8, 4 (g % 2) + l / 8, g / 2)
+            const unsigned mx = __shfl_sync(FULL, f, lane & 7u);
+            const unsigned m0 = mx & __shfl_sync(FULL, f, 8u + (lane >> 3));
+            const unsigned m1 = mx & __shfl_sync(FULL, f, 12u + (lane >> 3));
+#pragma unroll
+            for (int z = 0; z < 8; ++z) {
+                const unsigned mz = __shfl_sync(FULL, f, 16 + z);
+                cnt[2 * z] += __popc(m0 & mz);
+                cnt[2 * z + 1] += __popc(m1 & mz);
+            }
+        } else {
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) {
+                if (g < ngroups) {
+                    const unsigned c = 32u * g + lane;
+                    const unsigned mx = __shfl_sync(FULL, f, c & ((1u << d.lx) - 1u));
+                    const unsigned my = __shfl_sync(FULL, f, fy + ((c >> d.lx) & ((1u << d.ly) - 1u)));
+                    const unsigned mz = __shfl_sync(FULL, f, (fz + (c >> (d.lx + d.ly))) & 31u);
+                    cnt[g] += __popc(mx & my & mz);
+                }
+            }
+        }
+    }
+}
+
+// A warp per item.  A brick in one item writes its cells' counts; a chunk
+// writes its own to its slot, and the last chunk of the brick to arrive turns
+// the slots into offsets inside each cell and writes the sums.
+__global__ void __launch_bounds__(32 * COUNT_WARPS, 8) brick_count_kernel(BrickArgs a)
+{
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned nitems = min(ld_relaxed_u32(&a.ctl->tickets[3]), a.max_items);
+    const unsigned nempty = min(ld_relaxed_u32(&a.ctl->tickets[6]), a.max_items);
+    for (unsigned i = blockIdx.x * COUNT_WARPS + (threadIdx.x >> 5); i < nitems + nempty; i += gridDim.x * COUNT_WARPS) {
+        const BrickItem it = load_item(a.items + (i < nitems ? i : a.max_items - 1u - (i - nitems)));
+        const Dims d = decode(it.dims);
+        unsigned cnt[GROUPS];
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) cnt[g] = 0u;
+        count_words(a, it, d, cnt);
+        if (it.slot != NO_SLOT) {
+            unsigned *sl = a.slots + (size_t)it.slot * BRICK_CELLS;
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) sl[32 * g + lane] = cnt[g];
+            const uint2 meta = a.slot_meta[it.slot];
+            __threadfence();
+            __syncwarp();
+            unsigned last = 0u;
+            if (lane == 0u) last = atomicAdd(a.arrive + meta.x, 1u) + 1u == meta.y;
+            if (!__shfl_sync(FULL, last, 0)) continue;
+            __threadfence();
+            // every chunk of the brick is counted: offsets of the chunks inside each cell
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) cnt[g] = 0u;
+            for (unsigned j = 0; j < meta.y; ++j) {
+                unsigned *sj = a.slots + (size_t)(meta.x + j) * BRICK_CELLS;
+                unsigned v[GROUPS];
+#pragma unroll
+                for (int g = 0; g < GROUPS; ++g) v[g] = __ldcg(sj + 32 * g + lane);
+#pragma unroll
+                for (int g = 0; g < GROUPS; ++g) {
+                    sj[32 * g + lane] = cnt[g];
+                    cnt[g] += v[g];
+                }
+            }
+        }
+unsigned most = 0u;
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) most = max(most, cnt[g]);
+        const bool big = most >= BRICK_BIG;
+        if (d.nx == 8u && d.ny == 8u && d.nz == 8u && !big) {   // a whole cube: steps of 4 rows and of a layer
+            unsigned short *p = a.counts + (it.cell0 + (lane & 7u) + it.rx * (lane >> 3));
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g)
+                p[(size_t)(g & 1) * (4u * it.rx) + (size_t)(g >> 1) * it.rxy] = (unsigned short)cnt[g];
+            continue;
+        }
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) {
+            const unsigned c = 32u * g + lane;
+            const unsigned x = c & ((1u << d.lx) - 1u), y = (c >> d.lx) & ((1u << d.ly) - 1u), z = c >> (d.lx + d.ly);
+            if (x < d.nx && y < d.ny && z < d.nz) {
+                const unsigned cell = it.cell0 + x + it.rx * y + it.rxy * z;
+                a.counts[cell] = (unsigned short)min(cnt[g], BRICK_BIG);
+                if (cnt[g] >= BRICK_BIG) {
+                    const unsigned k = atomicAdd(&a.ctl->tickets[1], 1u);
+                    if (k < a.max_big)
+                        a.big[k] = make_uint2(cell, cnt[g]);
+                    else
+                        atomicOr(&a.ctl->err, ERR_RANGE);   // never: a cell of the list holds 65,535 pairs
+                }
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// scan: counts -> G
+// ---------------------------------------------------------------------------
+
+// Exclusive sums of the counts into the cells array.  A warp takes 256 J
+// consecutive cells in J coalesced 16-byte loads per lane.  In a batch each
+// mesh's slice ends in one word more than its cells (counted 0, so it gets the
+// mesh's total) and the sums are less the mesh's first pair; a single mesh is
+// a batch of one.
+//
+// Up to SCAN_ONE_PASS cells: one pass, look-back between tiles.  Beyond, the
+// look-back's chain would set the time (32 tiles per round trip): a first
+// pass adds up each tile, its last block scans the sums, a second pass reads
+// the counts again, half of them from L2.
+constexpr int SCAN_BLOCK = 256;
+constexpr int SCAN_WARPS = SCAN_BLOCK / 32;
+constexpr long long SCAN_ONE_PASS = 1ll << 20;
+constexpr int SCAN_J = 4;   // loads per lane of the two passes
+constexpr long long SCAN_TILE = (long long)SCAN_BLOCK * 8 * SCAN_J;
+constexpr long long SCAN_SMALL_TILE = (long long)SCAN_BLOCK * 8;
+
+struct Counts8 {
+    unsigned v[8];
+};
+
+// Mesh holding word p of the cells array (the last m with cells_off[m] <= p).
+__device__ __forceinline__ int mesh_of_word(const BrickArgs &a, long long p)
+{
+    int lo = 0, hi = a.mt.nm - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (__ldg(a.cells_off + mid) <= p)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    return lo;
+}
+
+__device__ __noinline__ unsigned big_count(const BrickArgs &a, unsigned cell)
+{
+    const unsigned n = min(ld_relaxed_u32(&a.ctl->tickets[1]), a.max_big);
+    for (unsigned k = 0; k < n; ++k) {
+        const uint2 e = a.big[k];
+        if (e.x == cell) return e.y;
+    }
+    return 0u;
+}
+
+// The 16-bit counts of words p .. p + 7 (p a multiple of 8) as they lie in
+// memory, zero beyond the last word.
+__device__ __forceinline__ uint4 load_raw(const BrickArgs &a, long long p)
+{
+    if (p + 8 <= a.ncells_out) return __ldcg(reinterpret_cast<const uint4 *>(a.counts + p));
+    unsigned w[4] = {0u, 0u, 0u, 0u};
+    for (int k = 0; k < 8; ++k)
+        if (p + k < a.ncells_out) w[k >> 1] |= (unsigned)__ldcg(a.counts + p + k) << (16 * (k & 1));
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// The eight counts: zero at the end of a mesh's slice, the list's value for a
+// cell of BRICK_BIG objects or more.  *m: a mesh at or before word p's on
+// entry (batched), word p's on return.
+__device__ __forceinline__ Counts8 unpack(const BrickArgs &a, const uint4 &q, long long p, int *m)
+{
+    Counts8 c;
+    const long long n = a.ncells_out;
+    const unsigned w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        c.v[2 * k] = w[k] & 0xFFFFu;
+        c.v[2 * k + 1] = w[k] >> 16;
+    }
+    if (a.mt.md) {
+        if (p < n) {
+            int s = *m;
+            long long end = __ldg(a.cells_off + s + 1);
+            while (end <= p) end = __ldg(a.cells_off + ++s + 1);
+            *m = s;
+            if (end <= p + 8) {   // a slice ends among the eight words
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    if (p + k < n) {
+                        while (end <= p + k) end = __ldg(a.cells_off + ++s + 1);
+                        if (p + k + 1 == end) c.v[k] = 0u;
+                    }
+                }
+            }
+        }
+    } else if (p + 8 >= n) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (p + k + 1 >= n) c.v[k] = 0u;
+    }
+    const unsigned ones = (__vcmpeq2(w[0], 0xFFFFFFFFu) | __vcmpeq2(w[1], 0xFFFFFFFFu)) |
+                          (__vcmpeq2(w[2], 0xFFFFFFFFu) | __vcmpeq2(w[3], 0xFFFFFFFFu));
+    if (ones) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (c.v[k] == BRICK_BIG) c.v[k] = big_count(a, (unsigned)(p + k));
+    }
+    return c;
+}
+
+__device__ __forceinline__ unsigned sum8(const Counts8 &c)
+{
+    return ((c.v[0] + c.v[1]) + (c.v[2] + c.v[3])) + ((c.v[4] + c.v[5]) + (c.v[6] + c.v[7]));
+}
+
+// G of words p .. p + 7 from the sum x before them.
+__device__ __forceinline__ void store_offsets(const BrickArgs &a, long long p, const Counts8 &c, unsigned x, int m)
+{
+    unsigned o[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        o[k] = x;
+        x += c.v[k];
+    }
+    if (a.mt.md && p < a.ncells_out) {
+        long long end = __ldg(a.cells_off + m + 1);
+        unsigned base = __ldg(a.pair_base + m);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (p + k < a.ncells_out) {
+                while (end <= p + k) {
+                    end = __ldg(a.cells_off + ++m + 1);
+                    base = __ldg(a.pair_base + m);
+                }
+                o[k] -= base;
+            }
+        }
+    }
+    if (p + 8 <= a.ncells_out) {
+        uint4 *g = reinterpret_cast<uint4 *>(a.G + p);
+        g[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        g[1] = make_uint4(o[4], o[5], o[6], o[7]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (p + k < a.ncells_out) a.G[p + k] = o[k];
+    }
+}
+
+// First pass: the sum of every tile; the last block to finish turns the sums
+// into offsets.
+__global__ void __launch_bounds__(SCAN_BLOCK) cell_sums_kernel(BrickArgs a, unsigned ntiles)
+{
+    __shared__ unsigned s_warp[SCAN_WARPS];
+    __shared__ unsigned s_last;
+    unsigned *sums = reinterpret_cast<unsigned *>(a.status);
+    const unsigned tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
+    const long long p0 = (long long)blockIdx.x * SCAN_TILE + (long long)w * (256 * SCAN_J) + 8 * lane;
+    uint4 raw[SCAN_J];
+#pragma unroll
+    for (int j = 0; j < SCAN_J; ++j) raw[j] = load_raw(a, p0 + 256 * j);
+    unsigned sum = 0u;
+    int m = a.mt.md ? mesh_of_word(a, p0) : 0;
+#pragma unroll
+    for (int j = 0; j < SCAN_J; ++j) sum += sum8(unpack(a, raw[j], p0 + 256 * j, &m));
+    sum = __reduce_add_sync(FULL, sum);
+    if (lane == 0u) s_warp[w] = sum;
+    __syncthreads();
+    if (tid == 0u) {
+        unsigned t = 0u;
+#pragma unroll
+        for (int k = 0; k < SCAN_WARPS; ++k) t += s_warp[k];
+        sums[blockIdx.x] = t;
+        __threadfence();
+        s_last = atomicAdd(&a.ctl->tickets[5], 1u) + 1u == gridDim.x;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    unsigned carry = 0u;
+    for (unsigned c0 = 0; c0 < ntiles; c0 += 4u * SCAN_BLOCK) {
+        const unsigned i = c0 + 4u * tid;
+        unsigned v[4];
+#pragma unroll
+        for (unsigned k = 0; k < 4u; ++k) v[k] = i + k < ntiles ? __ldcg(sums + i + k) : 0u;
+        unsigned total;
+        unsigned x = carry + block_excl_sum<SCAN_BLOCK>(v[0] + v[1] + v[2] + v[3], s_warp, &total);
+#pragma unroll
+        for (unsigned k = 0; k < 4u; ++k) {
+            if (i + k < ntiles) sums[i + k] = x;
+            x += v[k];
+        }
+        carry += total;
+    }
+}
+
+// The scan of one tile, from the first pass's offset or (LOOKBACK) from the
+// tiles before it.
+template <int J, bool LOOKBACK>
+__global__ void __launch_bounds__(SCAN_BLOCK) cell_scan_kernel(BrickArgs a)
+{
+    __shared__ unsigned s_tile;
+    __shared__ unsigned s_warp[SCAN_WARPS];
+    __shared__ unsigned s_excl;
+    const unsigned tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
+    unsigned tile = blockIdx.x;
+    if (LOOKBACK) {   // tiles in ticket order, so every tile a look-back waits for has started
+        if (tid == 0u) s_tile = atomicAdd(&a.ctl->tickets[5], 1u);
+        __syncthreads();
+        tile = s_tile;
+    }
+    const long long p0 = (long long)tile * (SCAN_BLOCK * 8 * J) + (long long)w * (256 * J) + 8 * lane;
+    uint4 raw[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) raw[j] = load_raw(a, p0 + 256 * j);
+    const int m0 = a.mt.md ? mesh_of_word(a, p0) : 0;
+    unsigned off[J];   // words of the warp before this lane's load j
+    unsigned run = 0u;
+    int m = m0;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const unsigned sum = sum8(unpack(a, raw[j], p0 + 256 * j, &m)), inc = warp_incl_sum(sum);
+        off[j] = run + inc - sum;
+        run += __shfl_sync(FULL, inc, 31);
+    }
+    if (lane == 31u) s_warp[w] = run;
+    __syncthreads();
+    if (w == 0u) {
+        const unsigned x = lane < (unsigned)SCAN_WARPS ? s_warp[lane] : 0u;
+        const unsigned inc = warp_incl_sum(x);
+        if (lane < (unsigned)SCAN_WARPS) s_warp[lane] = inc - x;
+        if (LOOKBACK) {
+            const unsigned total = __shfl_sync(FULL, inc, SCAN_WARPS - 1);
+            const unsigned long long excl = warp_lookback64(a.status, tile, total, a.ctl);
+            if (lane == 0u) s_excl = (unsigned)excl;
+        } else if (lane == 0u) {
+            s_excl = __ldg(reinterpret_cast<const unsigned *>(a.status) + tile);
+        }
+    }
+    __syncthreads();
+    const unsigned base = s_excl + s_warp[w];
+    m = m0;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        const Counts8 c = unpack(a, raw[j], p0 + 256 * j, &m);
+        store_offsets(a, p0 + 256 * j, c, base + off[j], m);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// fill: refs
+// ---------------------------------------------------------------------------
+
+constexpr unsigned MASK_PITCH = 36;   // words a row of 32 masks: rows of different words in different banks
+constexpr int FILL_WARPS = 4;         // a warp per 128 cells of the brick
+static_assert(BRICK_CHUNK <= 1024, "10 bits of entry in a tag");
+static_assert(BRICK_CELLS == FILL_WARPS * 128, "four cells per lane");
+
+// Stages the entries of words [q0, q1) that cover the lane's four cells, as
+// 16-bit tags: each cell's from its own position p on.  The four cells' lists
+// grow together, so finding an entry's bit is paid once for the cells it
+// covers.  A tag is `owner` over the entry; PER_CELL adds the cell of the four.
+template <bool PER_CELL>
+__device__ __forceinline__ void stage_entries(unsigned short *stage, const unsigned *mx, const unsigned *my,
+                                              const unsigned *mz, unsigned q0, unsigned q1, unsigned owner,
+                                              unsigned (&p)[4])
+{
+    for (unsigned q = q0; q < q1; ++q) {
+        const uint4 X = *reinterpret_cast<const uint4 *>(mx + MASK_PITCH * q);
+        const unsigned yz = my[MASK_PITCH * q] & mz[MASK_PITCH * q];
+        const unsigned m[4] = {X.x & yz, X.y & yz, X.z & yz, X.w & yz};
+        unsigned u = m[0] | m[1] | m[2] | m[3];
+        const unsigned tag = owner | (q << 5);
+        while (u) {
+            const unsigned b = __clz(u), t = 0x80000000u >> b;
+            u &= ~t;
+            const unsigned v = tag | b;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (m[i] & t) {
+                    stage[p[i]] = (unsigned short)(PER_CELL ? v | (unsigned)(i << 10) : v);
+                    ++p[i];
+                }
+            }
+        }
+    }
+}
+
+// A block per item, a warp per 128 cells, four neighbours in x per lane.  Of
+// every four rows each warp takes another one, skewed from layer to layer: a
+// surface that follows a plane of the brick keeps all warps busy.  The
+// pairs are staged in shared memory in output order, as (cells,
+// entry) in 16 bits, and copied out as objects with consecutive lanes on
+// consecutive refs (the cells of a row of the brick are neighbours in refs
+// too).  128 cells go at once when their pairs fit the stage, else 32 cells at
+// a time, four lanes per four cells with a quarter of the entries each, and
+// where 32 cells do not fit either, in windows of entries.
+template <unsigned STAGE, int MIN_BLOCKS>
+__global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel(BrickArgs a)
+{
+    static_assert(STAGE >= 1024, "one word of 32 cells fits");
+    constexpr unsigned W = FILL_WARPS;
+    __shared__ __align__(16) unsigned s_mask[BRICK_CHUNK / 32 * MASK_PITCH];   // [word of 32 entries][feature]
+    __shared__ unsigned s_obj[BRICK_CHUNK];
+    __shared__ unsigned short s_stage[W][STAGE];
+    __shared__ unsigned s_delta[W][32];                      // per cell: its refs' place less its staged place
+    const unsigned lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    const unsigned nitems = min(ld_relaxed_u32(&a.ctl->tickets[3]), a.max_items);
+    unsigned short *stage = s_stage[w];
+    unsigned *sdelta = s_delta[w];
+    bool bad = false;
+    for (unsigned i = blockIdx.x; i < nitems; i += gridDim.x) {
+        const BrickItem it = load_item(a.items + i);
+        const Dims d = decode(it.dims);
+        const unsigned nw = (it.count + 31u) >> 5;
+        Entry next = load_entry(a, it.first + 32u * w, 32u * w < it.count ? it.count - 32u * w : 0u);
+        // the lane's four cells: where each one's refs start and, of a brick in
+        // one item, how many it has; loaded ahead of the masks
+        const unsigned rr = 4u * (lane >> (d.lx - 2u)), row = rr + ((w + 2u * (rr >> d.ly)) & 3u);
+        const unsigned x = 4u * (lane & ((1u << (d.lx - 2u)) - 1u)), y = row & ((1u << d.ly) - 1u), z = row >> d.ly;
+        const unsigned c0 = (row << d.lx) + x;
+        unsigned dst[4], num[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dst[k] = num[k] = 0u;
+        if (y < d.ny && z < d.nz) {
+            const unsigned *gp = a.G + it.cell0 + x + it.rx * y + it.rxy * z;
+            unsigned g[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) g[k] = x + k <= d.nx ? __ldg(gp + k) : 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (x + k < d.nx) {
+                    dst[k] = it.base + g[k];
+                    num[k] = g[k + 1] - g[k];
+                    // the cell's other chunks come first; this one's share is counted below
+                    if (it.slot != NO_SLOT) dst[k] += __ldg(a.slots + (size_t)it.slot * BRICK_CELLS + c0 + k);
+                }
+            }
+        }
+        __syncthreads();   // the previous item's masks and objects are read
+        for (unsigned q = w; q < nw; q += W) {
+            const Entry cur = next;
+            const unsigned en = 32u * (q + W);
+            next = load_entry(a, it.first + en, en < it.count ? it.count - en : 0u);
+            s_mask[MASK_PITCH * q + lane] = transpose32(cur.ok ? feature_row(entry_info(a, cur), d) : 0u);
+            s_obj[32u * q + 31u - lane] = entry_obj(a, cur);
+        }
+        __syncthreads();
+        const unsigned fy = 1u << d.lx, fz = fy + (1u << d.ly);
+        const unsigned lsum = num[0] + num[1] + num[2] + num[3];
+        const unsigned inc = warp_incl_sum(lsum);
+        const unsigned total = __shfl_sync(FULL, inc, 31);
+        if (total == 0u) continue;
+        if (total <= STAGE && it.slot == NO_SLOT) {
+            unsigned p[4] = {inc - lsum, 0u, 0u, 0u};
+#pragma unroll
+            for (int k = 1; k < 4; ++k) p[k] = p[k - 1] + num[k - 1];
+            const unsigned delta = dst[0] - p[0];   // the lane's cells follow one another in refs as in the stage
+            if (lsum)
+                stage_entries<false>(stage, s_mask + x, s_mask + fy + y, s_mask + fz + z, 0u, nw, lane << 10, p);
+            bad |= p[3] != inc;
+            __syncwarp();
+            for (unsigned p0 = 0; p0 < total; p0 += 32u) {
+                const unsigned q = p0 + lane;
+                const unsigned v = q < total ? stage[q] : 0u;
+                const unsigned r = q + __shfl_sync(FULL, delta, v >> 10);
+                if (q < total) {
+                    if (r < a.nrefs)
+                        __stcs(a.refs + r, s_obj[v & 1023u]);
+                    else
+                        bad = true;
+                }
+            }
+            __syncwarp();
+            continue;
+        }
+        const unsigned quad = lane & 7u, sub = lane >> 3;
+        for (unsigned g = 0; g < 4u; ++g) {
+            // cells 32 g .. 32 g + 31 of the warp's: those of lanes 8 g .. 8 g + 7
+            const unsigned from = 8u * g + quad;
+            unsigned to[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) to[k] = __shfl_sync(FULL, dst[k], from);
+            const bool live = __shfl_sync(FULL, lsum, from) != 0u;   // a cell beyond a small brick has no features
+            if (!__any_sync(FULL, live)) continue;
+            const unsigned qx = __shfl_sync(FULL, x, from), qy = __shfl_sync(FULL, y, from),
+                           qz = __shfl_sync(FULL, z, from);
+            const unsigned *mx = s_mask + qx, *my = s_mask + fy + qy, *mz = s_mask + ((fz + qz) & 31u);
+            unsigned win = nw;
+            for (unsigned q0 = 0; q0 < nw;) {
+                unsigned nq = min(win, nw - q0), qa, qb, k[4], pre[4], sum[4], base, cnt;
+                for (;;) {
+                    qa = q0 + nq * sub / 4u;
+                    qb = q0 + nq * (sub + 1u) / 4u;
+                    k[0] = k[1] = k[2] = k[3] = 0u;
+                    if (live) {
+                        for (unsigned q = qa; q < qb; ++q) {
+                            const uint4 X = *reinterpret_cast<const uint4 *>(mx + MASK_PITCH * q);
+                            const unsigned yz = my[MASK_PITCH * q] & mz[MASK_PITCH * q];
+                            k[0] += __popc(X.x & yz);
+                            k[1] += __popc(X.y & yz);
+                            k[2] += __popc(X.z & yz);
+                            k[3] += __popc(X.w & yz);
+                        }
+                    }
+                    // each cell's entries of the lower quarters, its sum, and the cells before
+                    unsigned all = 0u;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        unsigned v = k[j];
+                        const unsigned v1 = __shfl_up_sync(FULL, v, 8);
+                        if (sub >= 1u) v += v1;
+                        const unsigned v2 = __shfl_up_sync(FULL, v, 16);
+                        if (sub >= 2u) v += v2;
+                        pre[j] = v - k[j];
+                        sum[j] = __shfl_sync(FULL, v, 24u + quad);
+                        all += sum[j];
+                    }
+                    unsigned v = all;
+#pragma unroll
+                    for (int o = 1; o < 8; o <<= 1) {
+                        const unsigned t = __shfl_up_sync(FULL, v, o, 8);
+                        if (quad >= (unsigned)o) v += t;
+                    }
+                    base = v - all;
+                    cnt = __shfl_sync(FULL, v, 7);
+                    if (cnt <= STAGE) break;
+                    win = nq = nq / 2u;   // one word always fits
+                }
+                unsigned p[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    p[j] = base + pre[j];
+                    if (sub == 0u) sdelta[4u * quad + j] = to[j] - base;
+                    base += sum[j];
+                    to[j] += sum[j];
+                }
+                if (live) stage_entries<true>(stage, mx, my, mz, qa, qb, quad << 12, p);
+                __syncwarp();
+                for (unsigned p0 = lane; p0 < cnt; p0 += 32u) {
+                    const unsigned v = stage[p0];
+                    const unsigned r = p0 + sdelta[v >> 10];
+                    if (r < a.nrefs)
+                        __stcs(a.refs + r, s_obj[v & 1023u]);
+                    else
+                        bad = true;
+                }
+                __syncwarp();
+                q0 += nq;
+            }
+        }
+    }
+    if (bad) atomicOr(&a.ctl->err, ERR_RANGE);
+}
+
+// ---------------------------------------------------------------------------
+// launchers
+// ---------------------------------------------------------------------------
+
+// A brick in k > 1 chunks holds more than (k - 1) BRICK_CHUNK entries, at least
+// k BRICK_CHUNK / 2.
+unsigned brick_max_slots(unsigned count) { return 2u * (count / BRICK_CHUNK) + 2u; }
+
+unsigned brick_max_items(unsigned nbricks, unsigned count)
+{
+    const unsigned long long n = (unsigned long long)nbricks + brick_max_slots(count);
+    return n > 0xFFFFFFFFull ? 0xFFFFFFFFu : (unsigned)n;
+}
+
+unsigned long long cell_scan_tiles(long long ncells_out)
+{
+    const long long t = ncells_out > SCAN_ONE_PASS ? SCAN_TILE : SCAN_SMALL_TILE;
+    return (unsigned long long)((ncells_out + t - 1) / t);
+}
+
+cudaError_t launch_brick_split(const BrickArgs &a, cudaStream_t s)
+{
+    brick_split_kernel<<<(a.nbricks + 255u) / 256u, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s)
+{
+    const unsigned blocks = (a.max_items + COUNT_WARPS - 1u) / COUNT_WARPS, cap = (unsigned)nsm * 64u;
+    brick_count_kernel<<<blocks < cap ? blocks : cap, 32 * COUNT_WARPS, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s)
+{
+    const unsigned tiles = (unsigned)cell_scan_tiles(a.ncells_out);
+    if (a.ncells_out > SCAN_ONE_PASS) {
+        cell_sums_kernel<<<tiles, SCAN_BLOCK, 0, s>>>(a, tiles);
+        cell_scan_kernel<SCAN_J, false><<<tiles, SCAN_BLOCK, 0, s>>>(a);
+    } else {
+        cell_scan_kernel<1, true><<<tiles, SCAN_BLOCK, 0, s>>>(a);
+    }
+    return cudaGetLastError();
+}
+
+// Beyond 4 pairs per cell the larger stage wins, below the more resident blocks:
+// 165 against 225 us on the soup of 1M triangles (19 pairs per cell), 812
+// against 724 us on the building of 10M (2.4).
+constexpr double DENSE_PAIRS_PER_CELL = 4.0;
+
+cudaError_t launch_brick_fill(const BrickArgs &a, int nsm, cudaStream_t s)
+{
+    const unsigned cap = (unsigned)nsm * 64u, grid = a.max_items < cap ? a.max_items : cap;
+    if ((double)a.nrefs > DENSE_PAIRS_PER_CELL * (double)a.ncells_out)
+        brick_fill_kernel<2560, 8><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+    else
+        brick_fill_kernel<1024, 10><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace gg

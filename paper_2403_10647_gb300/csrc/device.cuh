@@ -17,6 +17,7 @@ constexpr unsigned ERR_RANGE = 16u;     // a key outside [0, ncells) or out of o
                                         // extraction, or a sort scatter fell outside the output
 constexpr unsigned ERR_TILE_REDO = 64u;        // not an error: count/scan could not record every pair
                                                // tile's first object; the host runs tile_search
+constexpr unsigned ERR_BTILE_REDO = 128u;      // not an error: the same for the brick entries' tiles
 constexpr unsigned ERR_LOCAL_FALLBACK = 32u;   // not an error: a group of buckets too large for the
                                                // per-bucket counting sort; the host places the build
                                                // by radix passes over every key bit instead
@@ -33,11 +34,14 @@ struct Ctl {
     unsigned hi_ord[3];         // atomicMax of ordered(max coordinate) per axis
     unsigned err;               // ERR_* bits
     unsigned spare;             // unused (keeps the layout)
-    unsigned long long nrefs;   // NO, written by the last count/scan tile
-    unsigned tickets[8];        // tile tickets: [0] count/scan, [7] culling emit; [2] counts the
-                                // hybrid placement's bucket groups
+    unsigned long long nrefs;   // NO, written by the last count/scan tile (with the brick entries in the
+                                // bits from BRICK_SUM_BITS on when it counted them)
+    unsigned tickets[8];        // tile tickets: [0] count/scan, [5] cell scan, [7] culling emit; counts: [1] cells of many objects,
+                                // [2] the hybrid placement's bucket groups, [3] the brick items,
+                                // [4] their chunk slots, [6] the empty bricks
     unsigned long long nkept;   // pairs the culling emit kept, written by its last tile
-    unsigned pad[4];
+    unsigned long long npairs;  // a count with brick entries: NO added up on its own, exact
+    unsigned pad[2];
     // grid metadata M computed on the device from the bounds above (plan_kernel),
     // for count/scan to read without a host round trip; the host checks it
     // against its own plan from the same bounds
@@ -78,6 +82,60 @@ __host__ __device__ __forceinline__ float ordered_to_float(unsigned k)
     __builtin_memcpy(&f, &b, 4);
     return f;
 #endif
+}
+
+// ---- bricks ----
+//
+// A brick is a box of 2^lx x 2^ly x 2^lz cells, at most 512.  A brick build
+// sorts one entry per (brick, object whose box meets it) instead of one pair
+// per cell; an entry carries the object's box inside the brick as two local
+// cell indices of 9 bits each.
+constexpr int BRICK_CELLS_LOG = 9;
+constexpr int BRICK_CELLS = 1 << BRICK_CELLS_LOG;
+constexpr int BRICK_INFO_BITS = 2 * BRICK_CELLS_LOG;
+// Count and scan of pairs and brick entries at once: one 62-bit sum holds the
+// pairs in its low BRICK_SUM_BITS bits and the entries above them (never more
+// than the pairs).  Whether the pairs overflowed shows in their own exact sum.
+constexpr int BRICK_SUM_BITS = 31;
+constexpr unsigned BRICK_SUM_MASK = (1u << BRICK_SUM_BITS) - 1u;
+
+__host__ __device__ __forceinline__ unsigned ceil_log2(unsigned v)
+{
+    unsigned b = 0;
+    while ((1u << b) < v) ++b;
+    return b;
+}
+
+// Brick shape of a grid, lx | ly << 4 | lz << 8: 8 cells along each axis, fewer
+// where the grid is thinner than that (in x at least 4, as the fill takes four
+// neighbours in x at a time); a thin grid's bricks are 16 cells
+// wide in x while the brick stays within 512 cells and its cell columns, rows
+// and layers within 32 (one bit each in a warp's 32 x 32 bit transpose).
+__host__ __device__ __forceinline__ unsigned brick_shape(int rx, int ry, int rz)
+{
+    unsigned cx = ceil_log2((unsigned)rx), cy = ceil_log2((unsigned)ry), cz = ceil_log2((unsigned)rz);
+    unsigned lx = cx < 2u ? 2u : cx < 3u ? cx : 3u, ly = cy < 3u ? cy : 3u, lz = cz < 3u ? cz : 3u;
+    if (cx > 3u && lx + ly + lz < (unsigned)BRICK_CELLS_LOG) lx = 4u;
+    return lx | (ly << 4) | (lz << 8);
+}
+
+// How a brick build's entries are packed into 32-bit keys and values: the
+// brick id in the key's low kb bits, the object in the value's low ob bits, the
+// box's BRICK_INFO_BITS in the bits above them (key first).
+struct BrickGen {
+    unsigned shape;      // single mesh: brick_shape, bricks per axis x and y
+    unsigned nbx, nby;
+    int kb, ob;
+};
+
+__host__ __device__ __forceinline__ int brick_key_info_bits(int kb)
+{
+    return 32 - kb < BRICK_INFO_BITS ? 32 - kb : BRICK_INFO_BITS;
+}
+
+__host__ __device__ __forceinline__ bool brick_packs(int kb, int ob)
+{
+    return ob + BRICK_INFO_BITS - brick_key_info_bits(kb) <= 32 && ob < 32 && kb < 32;
 }
 
 #ifdef __CUDACC__
@@ -134,6 +192,102 @@ __device__ __forceinline__ int cell_coord(float p, float lo, float scale, int re
     if (!(u >= 1.0f)) return 0;                 // u < 1 (incl. negative) or NaN
     if (u >= (float)res) return res - 1;        // floor(u) > res - 1
     return __float2int_rz(u);                   // u in [1, res): truncation == floor
+}
+
+// ---- block and grid primitives ----
+
+template <typename T>
+__device__ __forceinline__ T warp_incl_sum(T v)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        T u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    return v;
+}
+
+__device__ __forceinline__ unsigned warp_incl_max(unsigned v)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        unsigned u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v = max(v, u);
+    }
+    return v;
+}
+
+// Exclusive block-wide sum of one value per thread; s_tmp holds BLOCK/32
+// entries.  Returns the exclusive prefix, writes the block total to *total.
+template <int BLOCK, typename T>
+__device__ __forceinline__ T block_excl_sum(T v, T *s_tmp, T *total)
+{
+    constexpr int W = BLOCK / 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    T inc = warp_incl_sum(v);
+    if (lane == 31) s_tmp[w] = inc;
+    __syncthreads();
+    if (w == 0) {
+        T x = lane < W ? s_tmp[lane] : T(0);
+        x = warp_incl_sum(x);
+        if (lane < W) s_tmp[lane] = x;
+    }
+    __syncthreads();
+    T wex = w ? s_tmp[w - 1] : T(0);
+    *total = s_tmp[W - 1];
+    __syncthreads();
+    return wex + inc - v;
+}
+
+constexpr unsigned long long LB64_AGG = 1ull << 62;
+constexpr unsigned long long LB64_PREFIX = 2ull << 62;
+constexpr unsigned long long LB64_VALUE = (1ull << 62) - 1ull;
+
+// Decoupled look-back of tile t over 64-bit status words (flag | value), run
+// by one whole warp: publishes t's aggregate, reads 32 predecessors per round
+// trip (lane q reads tile k - q), adds every aggregate up to the nearest
+// inclusive prefix, then publishes t's own inclusive prefix.  A word not yet
+// published ahead of that prefix means polling the window again, at most
+// SPIN_LIMIT times (then ERR_TIMEOUT and the partial sum).  Returns the
+// exclusive prefix in every lane.
+__device__ __forceinline__ unsigned long long warp_lookback64(unsigned long long *st, unsigned t,
+                                                              unsigned long long total, Ctl *ctl)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned long long excl = 0;
+    if (t == 0) {
+        if (lane == 0) st_relaxed_u64(&st[0], LB64_PREFIX | total);
+        return 0ull;
+    }
+    if (lane == 0) st_relaxed_u64(&st[t], LB64_AGG | total);
+    long long k = (long long)t - 1;
+    unsigned spins = 0;
+    while (true) {
+        const long long idx = k - lane;
+        const unsigned long long v = idx >= 0 ? ld_relaxed_u64(&st[idx]) : LB64_PREFIX;
+        const unsigned pre = __ballot_sync(0xffffffffu, (v & LB64_PREFIX) != 0ull);
+        const unsigned zero = __ballot_sync(0xffffffffu, v == 0ull);
+        const int p = pre ? __ffs(pre) - 1 : 32;                // nearest prefix in the window
+        const unsigned upto = p < 31 ? (2u << p) - 1u : 0xffffffffu;
+        if (zero & upto) {                                       // a nearer tile has not published
+            if (++spins > SPIN_LIMIT) {
+                if (lane == 0) atomicOr(&ctl->err, ERR_TIMEOUT);
+                break;
+            }
+            if (spins > 8) __nanosleep(64);
+            continue;
+        }
+        unsigned long long part = lane <= p ? (v & LB64_VALUE) : 0ull;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+        excl += part;
+        if (p < 32) break;
+        k -= 32;
+    }
+    if (lane == 0) st_relaxed_u64(&st[t], LB64_PREFIX | ((excl + total) & LB64_VALUE));
+    return excl;
 }
 
 #endif  // __CUDACC__

@@ -45,51 +45,6 @@ namespace gg {
 // helpers
 // ---------------------------------------------------------------------------
 
-template <typename T>
-__device__ __forceinline__ T warp_incl_sum(T v)
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        T u = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += u;
-    }
-    return v;
-}
-
-__device__ __forceinline__ unsigned warp_incl_max(unsigned v)
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        unsigned u = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v = max(v, u);
-    }
-    return v;
-}
-
-// Exclusive block-wide sum of one value per thread; s_tmp holds BLOCK/32
-// entries.  Returns the exclusive prefix, writes the block total to *total.
-template <int BLOCK, typename T>
-__device__ __forceinline__ T block_excl_sum(T v, T *s_tmp, T *total)
-{
-    constexpr int W = BLOCK / 32;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    T inc = warp_incl_sum(v);
-    if (lane == 31) s_tmp[w] = inc;
-    __syncthreads();
-    if (w == 0) {
-        T x = lane < W ? s_tmp[lane] : T(0);
-        x = warp_incl_sum(x);
-        if (lane < W) s_tmp[lane] = x;
-    }
-    __syncthreads();
-    T wex = w ? s_tmp[w - 1] : T(0);
-    *total = s_tmp[W - 1];
-    __syncthreads();
-    return wex + inc - v;
-}
-
 // Shared-memory index with one pad word per 32: rows written in blocked
 // arrangement (thread t at t * ITEMS + i) and read warp-striped both hit 32
 // distinct banks.
@@ -105,7 +60,10 @@ __host__ __device__ constexpr int padded() { return T + T / 32; }
 // object of the thread's pair j0 + tid * ITEMS + i.  mark holds padded<T>()
 // entries and must be zero on entry (zero_marks, once per block); every
 // thread clears the entries it reads, so it is zero again on return and the
-// next tile needs no clearing pass.  s_tmp holds BLOCK / 32 entries.
+// next tile needs no clearing pass.  s_tmp holds BLOCK / 32 entries.  Object o
+// starts at starts[o * stride].
+constexpr unsigned REC_WORDS = sizeof(ObjRec) / sizeof(unsigned);
+
 template <int BLOCK, int ITEMS>
 __device__ __forceinline__ void zero_marks(unsigned *mark)
 {
@@ -113,7 +71,7 @@ __device__ __forceinline__ void zero_marks(unsigned *mark)
 }
 
 template <int BLOCK, int ITEMS>
-__device__ __forceinline__ unsigned tile_objects(const ObjRec *__restrict__ recs,
+__device__ __forceinline__ unsigned tile_objects(const unsigned *__restrict__ starts, unsigned stride,
                                                  const unsigned *__restrict__ tile_obj, unsigned t,
                                                  unsigned j0, unsigned cnt, unsigned *mark,
                                                  unsigned *s_tmp, unsigned (&om)[ITEMS])
@@ -122,7 +80,7 @@ __device__ __forceinline__ unsigned tile_objects(const ObjRec *__restrict__ recs
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const unsigned of = tile_obj[t], ol = tile_obj[t + 1];
     for (unsigned o = of + 1u + tid; o <= ol; o += BLOCK) {
-        const unsigned s = __ldg(&recs[o].start);
+        const unsigned s = __ldg(starts + (size_t)o * stride);
         const unsigned p = s - j0;
         if (s >= j0 && p < cnt) mark[pad32(p)] = o - of;
     }
@@ -233,6 +191,84 @@ __device__ __forceinline__ void gen_blocked(const ObjRec *__restrict__ recs, uns
     }
 }
 
+// The same for a brick build: the thread's ITEMS consecutive entries (brick,
+// object) of the tile, x fastest over the bricks that the object's box meets,
+// each packed with the part of the box inside the brick (BrickGen).
+template <int ITEMS>
+__device__ __forceinline__ void gen_bricks(const ObjRec *__restrict__ recs, const unsigned *__restrict__ bstart,
+                                           unsigned of, const unsigned (&om)[ITEMS], unsigned j0, unsigned cnt,
+                                           const BrickGen &bg, const MeshTab &mt, unsigned (&keys)[ITEMS],
+                                           unsigned (&objs)[ITEMS])
+{
+    const unsigned e0 = threadIdx.x * ITEMS;
+    const int ks = brick_key_info_bits(bg.kb);
+    unsigned o = 0u, x = 0u, y = 0u, z = 0u;
+    unsigned lo[3] = {0u, 0u, 0u}, hi[3] = {0u, 0u, 0u}, b0[3] = {0u, 0u, 0u}, b1[3] = {0u, 0u, 0u};
+    unsigned shape = bg.shape, nbx = bg.nbx, nby = bg.nby, kbase = 0u, obase = 0u;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const unsigned e = e0 + i;
+        keys[i] = 0u;
+        objs[i] = 0u;
+        if (e < cnt) {
+            const unsigned oe = of + om[i];
+            if (i == 0 || oe != o) {
+                o = oe;
+                const uint4 r = __ldg(reinterpret_cast<const uint4 *>(recs) + o);
+                if (mt.md) {
+                    const int m = mesh_of(mt, o);
+                    shape = __ldg(&mt.md[m].shape);
+                    nbx = __ldg(&mt.md[m].nbx);
+                    nby = __ldg(&mt.md[m].nby);
+                    kbase = __ldg(&mt.md[m].brick_base);
+                    obase = (unsigned)__ldg(mt.obj_base + m);
+                }
+                lo[0] = r.x & 0xFFFFu;
+                lo[1] = r.x >> 16;
+                lo[2] = r.y & 0xFFFFu;
+                hi[0] = r.y >> 16;
+                hi[1] = r.z & 0xFFFFu;
+                hi[2] = r.z >> 16;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const unsigned l = (shape >> (4 * a)) & 15u;
+                    b0[a] = lo[a] >> l;
+                    b1[a] = hi[a] >> l;
+                }
+                x = b0[0];
+                y = b0[1];
+                z = b0[2];
+                if (i == 0) {
+                    const unsigned rid = j0 + e - __ldg(bstart + o);
+                    const unsigned mx = b1[0] - b0[0] + 1u, mxy = mx * (b1[1] - b0[1] + 1u);
+                    if (rid) {
+                        const unsigned q = rid / mxy, rem = rid - q * mxy, p = rem / mx;
+                        z += q;
+                        y += p;
+                        x += rem - p * mx;
+                    }
+                }
+            } else if (++x > b1[0]) {
+                x = b0[0];
+                if (++y > b1[1]) {
+                    y = b0[1];
+                    ++z;
+                }
+            }
+            const unsigned lx = shape & 15u, ly = (shape >> 4) & 15u, lz = (shape >> 8) & 15u;
+            // the box inside the brick: its own faces in the first and last brick, the brick's else
+            const unsigned mx = (1u << lx) - 1u, my = (1u << ly) - 1u, mz = (1u << lz) - 1u;
+            const unsigned l0 = (x == b0[0] ? lo[0] & mx : 0u) | ((y == b0[1] ? lo[1] & my : 0u) << lx) |
+                                ((z == b0[2] ? lo[2] & mz : 0u) << (lx + ly));
+            const unsigned l1 = (x == b1[0] ? hi[0] & mx : mx) | ((y == b1[1] ? hi[1] & my : my) << lx) |
+                                ((z == b1[2] ? hi[2] & mz : mz) << (lx + ly));
+            const unsigned info = l0 | (l1 << BRICK_CELLS_LOG);
+            keys[i] = (kbase + x + nbx * (y + nby * z)) | (info << bg.kb);   // the key takes the low ks info bits
+            objs[i] = (o - obase) | ((info >> ks) << bg.ob);
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // a0: boxes + scene bounds
 // ---------------------------------------------------------------------------
@@ -304,65 +340,29 @@ __global__ void __launch_bounds__(256) bounds_kernel(const float *__restrict__ v
 // a2 + a3: CountCells + ExclusiveSum (single pass, decoupled look-back)
 // ---------------------------------------------------------------------------
 
-constexpr unsigned long long LB64_AGG = 1ull << 62;
-constexpr unsigned long long LB64_PREFIX = 2ull << 62;
-constexpr unsigned long long LB64_VALUE = (1ull << 62) - 1ull;
-
-// Decoupled look-back of tile t over 64-bit status words (flag | value), run
-// by one whole warp: publishes t's aggregate, reads 32 predecessors per round
-// trip (lane q reads tile k - q), adds every aggregate up to the nearest
-// inclusive prefix, then publishes t's own inclusive prefix.  A word not yet
-// published ahead of that prefix means polling the window again, at most
-// SPIN_LIMIT times (then ERR_TIMEOUT and the partial sum).  Returns the
-// exclusive prefix in every lane.
-__device__ __forceinline__ unsigned long long warp_lookback64(unsigned long long *st, unsigned t,
-                                                              unsigned long long total, Ctl *ctl)
-{
-    const int lane = threadIdx.x & 31;
-    unsigned long long excl = 0;
-    if (t == 0) {
-        if (lane == 0) st_relaxed_u64(&st[0], LB64_PREFIX | total);
-        return 0ull;
-    }
-    if (lane == 0) st_relaxed_u64(&st[t], LB64_AGG | total);
-    long long k = (long long)t - 1;
-    unsigned spins = 0;
-    while (true) {
-        const long long idx = k - lane;
-        const unsigned long long v = idx >= 0 ? ld_relaxed_u64(&st[idx]) : LB64_PREFIX;
-        const unsigned pre = __ballot_sync(0xffffffffu, (v & LB64_PREFIX) != 0ull);
-        const unsigned zero = __ballot_sync(0xffffffffu, v == 0ull);
-        const int p = pre ? __ffs(pre) - 1 : 32;                // nearest prefix in the window
-        const unsigned upto = p < 31 ? (2u << p) - 1u : 0xffffffffu;
-        if (zero & upto) {                                       // a nearer tile has not published
-            if (++spins > SPIN_LIMIT) {
-                if (lane == 0) atomicOr(&ctl->err, ERR_TIMEOUT);
-                break;
-            }
-            if (spins > 8) __nanosleep(64);
-            continue;
-        }
-        unsigned long long part = lane <= p ? (v & LB64_VALUE) : 0ull;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-        excl += part;
-        if (p < 32) break;
-        k -= 32;
-    }
-    if (lane == 0) st_relaxed_u64(&st[t], LB64_PREFIX | ((excl + total) & LB64_VALUE));
-    return excl;
-}
-
-template <int BLOCK, int ITEMS>
+// BRICKS: the bricks that an object's box meets are counted and scanned with
+// the pairs, in the bits from BRICK_SUM_BITS on, and the pairs added up once
+// more on their own, so that the host knows whether they overflowed theirs.
+template <int BLOCK, int ITEMS, bool BRICKS>
 __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(CountArgs a)
 {
     constexpr int T = BLOCK * ITEMS;
     __shared__ unsigned long long s_pref[T];
     __shared__ unsigned long long s_tmp[BLOCK / 32];
     __shared__ unsigned s_tile;
-    __shared__ unsigned long long s_excl;
+    __shared__ unsigned long long s_excl, s_pairs;
+    __shared__ int s_mesh0, s_mesh1;
     const int tid = threadIdx.x;
-    if (tid == 0) s_tile = atomicAdd(&a.ctl->tickets[0], 1u);
+    if (tid == 0) {
+        const unsigned t = atomicAdd(&a.ctl->tickets[0], 1u);
+        s_tile = t;
+        s_pairs = 0ull;
+        if (a.mt.md) {   // the meshes of the tile's first and last object
+            const long long o0 = (long long)t * T;
+            s_mesh0 = mesh_of(a.mt, o0);
+            s_mesh1 = mesh_of(a.mt, min(o0 + T, a.n) - 1);
+        }
+    }
     if (a.device_plan) {   // the plan kernel's M, in place of the host's
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
@@ -374,11 +374,14 @@ __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(Cou
     __syncthreads();
     const unsigned tile = s_tile;
     const long long base = (long long)tile * T;
+    const bool one_mesh = !a.mt.md || s_mesh0 == s_mesh1;
+    unsigned shape = BRICKS && !a.mt.md ? brick_shape(a.res[0], a.res[1], a.res[2]) : 0u;
+    unsigned long long pairs = 0ull;
 
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
         const long long o = base + i * BLOCK + tid;
-        unsigned V = 0u;
+        unsigned long long V = 0ull;
         if (o < a.n) {
             // the triangle and the grid it maps into: the single mesh's, or
             // in a batched build the owning mesh's
@@ -388,8 +391,9 @@ __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(Cou
             float glo[3] = {a.lo[0], a.lo[1], a.lo[2]}, gsc[3] = {a.scale[0], a.scale[1], a.scale[2]};
             int gres[3] = {a.res[0], a.res[1], a.res[2]};
             if (a.mt.md) {
-                const int m = mesh_of(a.mt, o);
+                const int m = one_mesh ? s_mesh0 : mesh_of(a.mt, o);
                 const MeshDesc &md = a.mt.md[m];
+                if (BRICKS) shape = md.shape;
                 tris = md.tris;
                 verts = md.verts;
                 nverts = md.nverts;
@@ -426,7 +430,17 @@ __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(Cou
             unsigned long long cnt = (unsigned long long)(chi[0] - clo[0] + 1u) *
                                      (unsigned long long)(chi[1] - clo[1] + 1u) *
                                      (unsigned long long)(chi[2] - clo[2] + 1u);
-            V = cnt > 0x80000000ull ? 0x80000000u : (unsigned)cnt;
+            V = cnt > 0x80000000ull ? 0x80000000ull : cnt;
+            if (BRICKS) {
+                pairs += V;
+                cnt = 1ull;
+#pragma unroll
+                for (int ax = 0; ax < 3; ++ax) {
+                    const unsigned l = (shape >> (4 * ax)) & 15u;
+                    cnt *= (unsigned long long)((chi[ax] >> l) - (clo[ax] >> l) + 1u);
+                }
+                V += (cnt > 0x80000000ull ? 0x80000000ull : cnt) << BRICK_SUM_BITS;
+            }
             // the box now, the pair offset once the scan has it: nothing
             // of the record stays live across the scan
             reinterpret_cast<uint4 *>(a.recs)[o] =
@@ -434,7 +448,13 @@ __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(Cou
         }
         s_pref[i * BLOCK + tid] = V;
     }
+    if (BRICKS) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) pairs += __shfl_xor_sync(0xffffffffu, pairs, off);
+        if ((tid & 31) == 0) atomicAdd(&s_pairs, pairs);
+    }
     __syncthreads();
+    if (BRICKS && tid == 0) atomicAdd(&a.ctl->npairs, s_pairs);
     unsigned long long run = 0;
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
@@ -451,43 +471,54 @@ __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(Cou
         const unsigned long long excl = warp_lookback64(a.status, tile, total, a.ctl);
         if (tid == 0) {
             s_excl = excl;
-            if (excl + total > 0x7FFFFFFFull) atomicOr(&a.ctl->err, ERR_OVERFLOW);
+            if (!BRICKS && excl + total > 0x7FFFFFFFull) atomicOr(&a.ctl->err, ERR_OVERFLOW);
             if (base + T >= a.n) a.ctl->nrefs = excl + total;
         }
     }
     __syncthreads();
     const unsigned long long excl = s_excl;
-    bool tile_redo = false;
+    bool tile_redo = false, btile_redo = false;
+    // the tiles whose first pair (or entry) is one of object o's [start, end):
+    // tile_search's answer, recorded here
+    auto record = [&](long long o, unsigned start, unsigned end, unsigned *tile_obj, unsigned cap, bool &redo) {
+        const unsigned t0 = (start + (unsigned)PAIR_TILE - 1u) / (unsigned)PAIR_TILE;
+        const unsigned tl = (end - 1u) / (unsigned)PAIR_TILE + 1u;   // tiles t0 .. tl - 1 (end > start)
+        if (tl <= cap && tl - t0 <= 64u) {
+            for (unsigned t = t0; t < tl; ++t) tile_obj[t] = (unsigned)o;
+        } else if (tl > t0) {
+            redo = true;
+        }
+        if (o == a.n - 1) {   // the entry after the last tile
+            const unsigned nt = (end + (unsigned)PAIR_TILE - 1u) / (unsigned)PAIR_TILE;
+            if (nt < cap) tile_obj[nt] = (unsigned)o; else redo = true;
+        }
+    };
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
         const int p = i * BLOCK + tid;
         const long long o = base + p;
         if (o < a.n) {
-            const unsigned start = (unsigned)(excl + s_pref[p]);
+            const unsigned long long at = excl + s_pref[p], next = excl + (p + 1 < T ? s_pref[p + 1] : total);
+            const unsigned start = BRICKS ? (unsigned)at & BRICK_SUM_MASK : (unsigned)at;
             a.recs[o].start = start;
             if (a.mt.md) {
-                const int m = mesh_of(a.mt, o);
+                const int m = one_mesh ? s_mesh0 : mesh_of(a.mt, o);
                 if (__ldg(a.mt.obj_base + m) == o) a.pair_base[m] = start;
             }
-            if (a.tile_obj && excl + total <= 0x7FFFFFFFull) {
-                // the pair tiles whose first pair is one of this object's
-                // [start, end): tile_search's answer, recorded here
-                const unsigned end = (unsigned)(excl + (p + 1 < T ? s_pref[p + 1] : total));
-                const unsigned t0 = (start + (unsigned)PAIR_TILE - 1u) / (unsigned)PAIR_TILE;
-                const unsigned tl = (end - 1u) / (unsigned)PAIR_TILE + 1u;   // tiles t0 .. tl - 1 (end > start)
-                if (tl <= a.tile_cap && tl - t0 <= 64u) {
-                    for (unsigned t = t0; t < tl; ++t) a.tile_obj[t] = (unsigned)o;
-                } else if (tl > t0) {
-                    tile_redo = true;
-                }
-                if (o == a.n - 1) {   // the entry after the last tile
-                    const unsigned nt = (end + (unsigned)PAIR_TILE - 1u) / (unsigned)PAIR_TILE;
-                    if (nt < a.tile_cap) a.tile_obj[nt] = (unsigned)o; else tile_redo = true;
-                }
+            if (BRICKS) {
+                const unsigned bs = (unsigned)(at >> BRICK_SUM_BITS);
+                a.bstart[o] = bs;
+                if (a.btile_obj)
+                    record(o, bs, (unsigned)(next >> BRICK_SUM_BITS), a.btile_obj, a.btile_cap, btile_redo);
+                if (a.tile_obj)
+                    record(o, start, (unsigned)next & BRICK_SUM_MASK, a.tile_obj, a.tile_cap, tile_redo);
+            } else if (a.tile_obj && excl + total <= 0x7FFFFFFFull) {
+                record(o, start, (unsigned)next, a.tile_obj, a.tile_cap, tile_redo);
             }
         }
     }
     if (tile_redo) atomicOr(&a.ctl->err, ERR_TILE_REDO);
+    if (BRICKS && btile_redo) atomicOr(&a.ctl->err, ERR_BTILE_REDO);
 }
 
 // ---------------------------------------------------------------------------
@@ -545,7 +576,7 @@ cudaError_t launch_plan(Ctl *ctl, long long n, float lambda, cudaStream_t s)
 // pair tiles: first object of each tile
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256) tile_search_kernel(const ObjRec *__restrict__ recs, long long n,
+__global__ void __launch_bounds__(256) tile_search_kernel(const unsigned *__restrict__ starts, int stride, long long n,
                                                           unsigned tile, unsigned ntiles,
                                                           unsigned *__restrict__ tile_obj)
 {
@@ -559,7 +590,7 @@ __global__ void __launch_bounds__(256) tile_search_kernel(const ObjRec *__restri
     long long lo = 0, hi = n - 1;
     while (lo < hi) {
         const long long mid = (lo + hi + 1) >> 1;
-        if (__ldg(&recs[mid].start) <= j)
+        if (__ldg(starts + mid * stride) <= j)
             lo = mid;
         else
             hi = mid - 1;
@@ -585,7 +616,7 @@ __global__ void __launch_bounds__(BLOCK) emit_kernel(EmitArgs a)
     zero_marks<BLOCK, ITEMS>(s_mark);
     __syncthreads();
     unsigned om[ITEMS];
-    const unsigned of = tile_objects<BLOCK, ITEMS>(a.recs, a.tile_obj, t, j0, cnt, s_mark, s_tmp, om);
+    const unsigned of = tile_objects<BLOCK, ITEMS>(&a.recs->start, REC_WORDS, a.tile_obj, t, j0, cnt, s_mark, s_tmp, om);
     unsigned keys[ITEMS], objs[ITEMS];
     gen_blocked<ITEMS>(a.recs, of, om, j0, cnt, a.res_x, a.res_y, a.mt, keys, objs);
     __syncthreads();
@@ -746,7 +777,7 @@ __global__ void __launch_bounds__(BLOCK) cull_emit_kernel(CullArgs a)
     __syncthreads();
     {
         unsigned om[ITEMS], keys[ITEMS], objs[ITEMS];
-        const unsigned of = tile_objects<BLOCK, ITEMS>(a.recs, a.tile_obj, t, j0, cnt, s_mark, s_tmp, om);
+        const unsigned of = tile_objects<BLOCK, ITEMS>(&a.recs->start, REC_WORDS, a.tile_obj, t, j0, cnt, s_mark, s_tmp, om);
         gen_blocked<ITEMS>(a.recs, of, om, j0, cnt, a.res_x, a.res_y, MeshTab{}, keys, objs);
         __syncthreads();   // every thread is done with the object marks
         // the thread's own items go to shared memory: the test loop below is
@@ -949,7 +980,7 @@ __host__ __device__ constexpr int gen_min_blocks()
 }
 
 template <int BLOCK, int ITEMS, int RBITS, int SRC>
-__global__ void __launch_bounds__(BLOCK, SRC == SRC_GEN ? gen_min_blocks<BLOCK>() : 2048 / BLOCK)
+__global__ void __launch_bounds__(BLOCK, SRC != SRC_MEM ? gen_min_blocks<BLOCK>() : 2048 / BLOCK)
     upsweep_kernel(UpArgs a)
 {
     constexpr int T = BLOCK * ITEMS;
@@ -964,7 +995,7 @@ __global__ void __launch_bounds__(BLOCK, SRC == SRC_GEN ? gen_min_blocks<BLOCK>(
     const unsigned t0 = g * a.gtiles, t1 = min(t0 + a.gtiles, a.ntiles);
     const unsigned sh = a.shift, mk = (1u << a.bits) - 1u;
     for (int i = tid; i < 3 * R; i += BLOCK) smem[i] = 0u;
-    if (SRC == SRC_GEN) zero_marks<BLOCK, ITEMS>(s_mark);
+    if (SRC != SRC_MEM) zero_marks<BLOCK, ITEMS>(s_mark);
     __syncthreads();
 
     // a tile's keys, 16 bytes per load where the whole run is in range and
@@ -997,10 +1028,15 @@ __global__ void __launch_bounds__(BLOCK, SRC == SRC_GEN ? gen_min_blocks<BLOCK>(
         const unsigned j0 = t * (unsigned)T;
         const unsigned cnt = min((unsigned)T, a.count - j0);
         unsigned *s_cnt = s_cnt2 + ((t - t0) & 1u) * R;
-        if (SRC == SRC_GEN) {
+        if (SRC != SRC_MEM) {
             unsigned om[ITEMS], objs[ITEMS];
-            const unsigned of = tile_objects<BLOCK, ITEMS>(a.recs, a.tile_obj, t, j0, cnt, s_mark, s_tmp, om);
-            gen_blocked<ITEMS>(a.recs, of, om, j0, cnt, a.res_x, a.res_y, a.mt, keys, objs);
+            const unsigned of = tile_objects<BLOCK, ITEMS>(SRC == SRC_BRICK ? a.bstart : &a.recs->start,
+                                                           SRC == SRC_BRICK ? 1u : REC_WORDS, a.tile_obj, t, j0, cnt,
+                                                           s_mark, s_tmp, om);
+            if (SRC == SRC_BRICK)
+                gen_bricks<ITEMS>(a.recs, a.bstart, of, om, j0, cnt, a.bg, a.mt, keys, objs);
+            else
+                gen_blocked<ITEMS>(a.recs, of, om, j0, cnt, a.res_x, a.res_y, a.mt, keys, objs);
             if (a.gen_keys) {
                 // store the object-order pairs once, for the first downsweep
                 // to read instead of generating them a second time
@@ -1217,7 +1253,7 @@ __global__ void __launch_bounds__(BLOCK, pass_min_blocks<BLOCK>()) downsweep_ker
         unsigned om[ITEMS], objs[ITEMS];
         zero_marks<BLOCK, ITEMS>(s_mark);
         __syncthreads();
-        const unsigned of = tile_objects<BLOCK, ITEMS>(a.recs, a.tile_obj, tile, j0, cnt, s_mark, s_tmp, om);
+        const unsigned of = tile_objects<BLOCK, ITEMS>(&a.recs->start, REC_WORDS, a.tile_obj, tile, j0, cnt, s_mark, s_tmp, om);
         gen_blocked<ITEMS>(a.recs, of, om, j0, cnt, a.res_x, a.res_y, a.mt, keys, objs);
         __syncthreads();
 #pragma unroll
@@ -2054,7 +2090,10 @@ cudaError_t launch_count_scan(const CountArgs &a, cudaStream_t s)
 {
     if (a.n <= 0) return cudaSuccess;
     const long long tiles = (a.n + COUNT_TILE - 1) / COUNT_TILE;
-    count_scan_kernel<COUNT_BLOCK, COUNT_TILE / COUNT_BLOCK><<<(unsigned)tiles, COUNT_BLOCK, 0, s>>>(a);
+    if (a.bricks)
+        count_scan_kernel<COUNT_BLOCK, COUNT_TILE / COUNT_BLOCK, true><<<(unsigned)tiles, COUNT_BLOCK, 0, s>>>(a);
+    else
+        count_scan_kernel<COUNT_BLOCK, COUNT_TILE / COUNT_BLOCK, false><<<(unsigned)tiles, COUNT_BLOCK, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -2073,11 +2112,11 @@ cudaError_t allow_dynamic_smem(K k, size_t smem, std::atomic<unsigned long long>
     return e;
 }
 
-cudaError_t launch_tile_search(const ObjRec *recs, long long n, unsigned tile, unsigned ntiles,
+cudaError_t launch_tile_search(const unsigned *starts, int stride, long long n, unsigned tile, unsigned ntiles,
                                unsigned *tile_obj, cudaStream_t s)
 {
     const unsigned blocks = (ntiles + 1 + 255) / 256;
-    tile_search_kernel<<<blocks, 256, 0, s>>>(recs, n, tile, ntiles, tile_obj);
+    tile_search_kernel<<<blocks, 256, 0, s>>>(starts, stride, n, tile, ntiles, tile_obj);
     return cudaGetLastError();
 }
 
@@ -2116,7 +2155,7 @@ static cudaError_t launch_up_t(const UpArgs &a, cudaStream_t s)
 {
     constexpr int ITEMS = PAIR_TILE / BLOCK;
     auto k = upsweep_kernel<BLOCK, ITEMS, RBITS, SRC>;
-    const size_t smem = sizeof(unsigned) * (3 * (1 << RBITS) + (SRC == SRC_GEN ? padded<PAIR_TILE>() : 0));
+    const size_t smem = sizeof(unsigned) * (3 * (1 << RBITS) + (SRC != SRC_MEM ? padded<PAIR_TILE>() : 0));
     static std::atomic<unsigned long long> configured{0};
     if (cudaError_t e = allow_dynamic_smem(k, smem, configured)) return e;
     if (a.gtiles < 1 || a.gtiles > (unsigned)GROUP_TILES) return cudaErrorInvalidValue;
@@ -2149,7 +2188,9 @@ static cudaError_t launch_up_b(const UpArgs &a, int rbits, int src, cudaStream_t
 {
 #define GG_UP(RB)                                                                                   \
     case RB:                                                                                        \
-        return src == SRC_GEN ? launch_up_t<RB, SRC_GEN, BLOCK>(a, s) : launch_up_t<RB, SRC_MEM, BLOCK>(a, s);
+        return src == SRC_GEN     ? launch_up_t<RB, SRC_GEN, BLOCK>(a, s)                               \
+               : src == SRC_BRICK ? launch_up_t<RB, SRC_BRICK, BLOCK>(a, s)                             \
+                                  : launch_up_t<RB, SRC_MEM, BLOCK>(a, s);
     switch (rbits) {
         GG_UP(8)
         GG_UP(9)

@@ -58,7 +58,7 @@ static_assert(GROUP_TILES * PAIR_TILE <= 65536, "tile offsets inside a group fit
 constexpr int EXTRACT_BLOCK = 256;
 constexpr int EXTRACT_TILE = 4096;
 
-enum { SRC_MEM = 0, SRC_GEN = 1 };
+enum { SRC_MEM = 0, SRC_GEN = 1, SRC_BRICK = 2 };
 
 // A batch of meshes built as one flattened problem: mesh m owns objects
 // [obj_base[m], obj_base[m + 1]) and global cell ids [cell_base,
@@ -73,6 +73,8 @@ struct MeshDesc {
     float scale[3];
     int res[3];
     unsigned cell_base;
+    unsigned shape, nbx, nby;       // brick builds: brick_shape, bricks along x and y,
+    unsigned brick_base;            // the mesh's first brick
 };
 
 struct MeshTab {
@@ -98,6 +100,10 @@ struct CountArgs {
     unsigned *tile_obj;             // single mesh, optional: [tile_cap] the first object of every
     unsigned tile_cap;              // PAIR_TILE-pair tile and, after the last tile, n - 1 (tile_search's
                                     // result), or ERR_TILE_REDO when it did not fit
+    bool bricks;                    // count and scan the brick entries too:
+    unsigned *bstart;               // [n] out: the exclusive prefix sum of the entries
+    unsigned *btile_obj;            // as tile_obj for tiles of PAIR_TILE entries, or ERR_BTILE_REDO
+    unsigned btile_cap;
 };
 
 struct EmitArgs {
@@ -137,7 +143,9 @@ struct UpArgs {
     const unsigned *tile_obj;       // SRC_GEN
     MeshTab mt;                     // SRC_GEN, batched
     unsigned res_x, res_y;          // SRC_GEN
-    unsigned *gen_keys;             // SRC_GEN: if set, the generated pairs are stored here
+    BrickGen bg;                    // SRC_BRICK
+    const unsigned *bstart;         // SRC_BRICK: first entry of each object
+    unsigned *gen_keys;             // SRC_GEN, SRC_BRICK: if set, the generated pairs are stored here
     unsigned *gen_vals;             //   (object order, [count] each) for the first downsweep
     unsigned count;
     unsigned ntiles;
@@ -224,8 +232,14 @@ cudaError_t launch_count_scan(const CountArgs &a, cudaStream_t s);
 // ctl->plan_*.  With an error bit already set it writes a harmless plan
 // (one cell, scale 0).
 cudaError_t launch_plan(Ctl *ctl, long long n, float lambda, cudaStream_t s);
-cudaError_t launch_tile_search(const ObjRec *recs, long long n, unsigned tile, unsigned ntiles,
+// starts[o * stride] = first pair (or entry) of object o.
+cudaError_t launch_tile_search(const unsigned *starts, int stride, long long n, unsigned tile, unsigned ntiles,
                                unsigned *tile_obj, cudaStream_t s);
+inline cudaError_t launch_tile_search(const ObjRec *recs, long long n, unsigned tile, unsigned ntiles,
+                                      unsigned *tile_obj, cudaStream_t s)
+{
+    return launch_tile_search(&recs->start, (int)(sizeof(ObjRec) / sizeof(unsigned)), n, tile, ntiles, tile_obj, s);
+}
 cudaError_t launch_emit(const EmitArgs &a, cudaStream_t s);
 cudaError_t launch_cull_emit(const CullArgs &a, cudaStream_t s);
 // Runs the look-back wait on col[0], which must be zero and stay zero.
@@ -284,6 +298,61 @@ struct LocalArgs {
 // G[ncells] = count; the first bucket of every group appended to groups.
 cudaError_t launch_bucket_split(const LocalArgs &a, cudaStream_t s);
 cudaError_t launch_local_sort(const LocalArgs &a, cudaStream_t s);
+
+// ---- brick builds (bricks.cu) ----
+//
+// The radix passes have ordered the entries by brick, objects ascending in
+// each.  split lists the bricks' entries as work items, count finds every
+// cell's number of objects, scan turns the numbers into G, fill writes the
+// object ids in cell order.
+constexpr int BRICK_CHUNK = 1024;   // entries per item
+
+// One brick's entries [first, first + count), or a chunk of them.
+struct __align__(32) BrickItem {
+    unsigned cell0;      // the brick's first cell in the output cells array
+    unsigned rx, rxy;    // cell steps to the next row and layer
+    unsigned first, count;
+    unsigned slot;       // of a brick in chunks: this chunk's slot, else 0xFFFFFFFF
+    unsigned dims;       // cells inside the grid - 1 per axis (5 bits each), lx, ly, lz (3 bits each)
+    unsigned base;       // first pair of the brick's mesh
+};
+
+struct BrickArgs {
+    const unsigned *keys, *vals;    // [count] entries ordered by brick
+    unsigned count;
+    int kb, ob;                     // packing (BrickGen)
+    unsigned nbricks;
+    // single mesh; batched: mt, cells_off, pair_base per mesh
+    int res[3];
+    unsigned shape, nbx, nby;
+    MeshTab mt;
+    const long long *cells_off;     // [nm + 1]
+    const unsigned *pair_base;      // [nm]
+    BrickItem *items;               // [max_items]: items from the front, empty bricks from the back
+    unsigned max_items;
+    unsigned max_slots;
+    unsigned *slots;                // [max_slots][BRICK_CELLS]: a chunk's counts, then its offsets in the cells
+    uint2 *slot_meta;               // [max_slots]: the brick's first slot and its number of slots
+    unsigned *arrive;               // [max_slots]: chunks counted, at the brick's first slot
+    unsigned short *counts;         // [ncells_out] objects per cell; BRICK_BIG and more: in `big`
+    uint2 *big;                     // [max_big]: cell, objects
+    unsigned max_big;
+    unsigned *G;                    // the output cells array(s), ncells_out words
+    long long ncells_out;
+    unsigned long long *status;     // [cell_scan_tiles] look-back words, zeroed, or tile sums
+    unsigned *refs;
+    unsigned nrefs;
+    Ctl *ctl;                       // tickets [1], [3] .. [6] zero on entry
+};
+constexpr unsigned BRICK_BIG = 65535u;
+
+unsigned brick_max_slots(unsigned count);
+unsigned brick_max_items(unsigned nbricks, unsigned count);
+unsigned long long cell_scan_tiles(long long ncells_out);
+cudaError_t launch_brick_split(const BrickArgs &a, cudaStream_t s);
+cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s);
+cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s);
+cudaError_t launch_brick_fill(const BrickArgs &a, int nsm, cudaStream_t s);
 
 unsigned long long extract_blocks(unsigned long long count, unsigned long long ncells);
 cudaError_t launch_extract_split(const ExtractArgs &a, cudaStream_t s);

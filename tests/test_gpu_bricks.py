@@ -1,0 +1,84 @@
+"""Brick builds: radix passes over (brick, object) entries, then per brick the
+objects of every cell (split, count, scan, fill).  Each grid equals the
+oracle's bit for bit where the bricks can go wrong: grids thinner than a
+brick along any axis, grids that end inside a brick, cells and bricks too
+crowded for one stage, bricks in many chunks, a cell beyond the 16-bit counts,
+and batches of such meshes."""
+import numpy as np
+import pytest
+
+import oracle
+import scenes
+
+from test_gpu_parity import assert_grid_equal, dev
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _soup(n, box, edge, seed, lam, giants=0, crowd=0):
+    """n triangles of edges up to `edge` in `box`, `giants` of which span the
+    whole box, and `crowd` tiny ones inside one cell, in random order."""
+    g = np.random.Generator(np.random.Philox(seed))
+    box = np.asarray(box, np.float64)
+    edge = np.minimum(edge, box)
+    c = g.random((n, 3)) * (box - edge)
+    v = np.stack([c, c + edge * g.random((n, 3)), c + edge * g.random((n, 3))], 1)
+    v[:giants] = np.stack([np.zeros(3), box, np.array([box[0], 0.0, box[2]])])
+    if crowd:
+        v = np.concatenate([v, np.broadcast_to(box * [0.503, 0.507, 0.511], (crowd, 3, 3))])
+    v = v[g.permutation(len(v))]
+    t = np.arange(3 * len(v), dtype=np.int32).reshape(-1, 3)
+    return scenes.Scene("bricks", v.reshape(-1, 3).astype(np.float32), t, lam)
+
+
+SCENES = {
+    # 8 x 8 x 8 bricks, ragged at every face, up to 100 objects per cell
+    "cube": lambda: _soup(30_000, (10, 9.3, 11.1), 2.5, 1, 4.0),
+    # thin and flat grids: other brick shapes
+    "thin_z": lambda: _soup(30_000, (60, 55, 0.9), 8.0, 2, 2.0),
+    "flat_z": lambda: _soup(20_000, (60, 55, 0), 9.0, 3, 4.0),
+    "flat_x": lambda: _soup(20_000, (0, 60, 55), 9.0, 4, 4.0),
+    "flat_y": lambda: _soup(20_000, (60, 0, 55), 9.0, 5, 4.0),
+    "line_x": lambda: _soup(20_000, (60, 0, 0), 3.0, 6, 2.0),
+    "line_z": lambda: _soup(20_000, (0, 0, 60), 3.0, 7, 2.0),
+    # every cell holds thousands: windows of entries, bricks in chunks
+    "few_cells": lambda: _soup(40_000, (1, 1.1, 0.9), 0.9, 8, 0.02),
+    # one cell of 70,000 objects: 16-bit counts are not enough
+    "big_cell": lambda: _soup(20_000, (10, 10, 10), 0.4, 9, 1.0, giants=60, crowd=70_000),
+}
+
+
+@pytest.mark.parametrize("name", sorted(SCENES))
+def test_brick_builds_match_oracle(name):
+    import paper_2403_10647_gb300 as pg
+    s = SCENES[name]()
+    o = oracle.build_grid(s.verts, s.tris, s.lam, method="counting")
+    c = pg.Context(0)
+    try:
+        c.profile(True)
+        for _ in range(2):   # the second build has the first one's buffers
+            g = c.build(dev(s.verts, torch.float32), dev(s.tris, torch.int32), s.lam)
+            assert_grid_equal(g, o, name)
+        assert "brick_count" in c.kernel_stats(), (o.NO, s.n)
+        if name == "big_cell":
+            assert np.diff(o.G).max() > 65_535
+    finally:
+        c.close()
+
+
+def test_brick_batch_matches_oracle():
+    import paper_2403_10647_gb300 as pg
+    empty = scenes.Scene("empty", np.zeros((0, 3), np.float32), np.zeros((0, 3), np.int32), 4.0)
+    batch = [empty, SCENES["thin_z"](), SCENES["big_cell"](), empty, _soup(3, (1, 2, 3), 0.5, 21, 8.0),
+             SCENES["flat_x"](), SCENES["line_z"](), empty]
+    c = pg.Context(0)
+    try:
+        c.profile(True)
+        grids = c.build_batched([(dev(s.verts, torch.float32), dev(s.tris, torch.int32), s.lam) for s in batch])
+        assert "brick_count" in c.kernel_stats()
+        for k, (s, g) in enumerate(zip(batch, grids)):
+            assert_grid_equal(g, oracle.build_grid(s.verts, s.tris, s.lam, method="counting"), f"mesh {k}")
+    finally:
+        c.close()
