@@ -20,7 +20,7 @@ BUILD_DIR = os.path.join(PKG_DIR, "_build")
 LIB_PATH = os.path.join(BUILD_DIR, "libgrid.so")
 
 SOURCES = ["kernels.cu", "bricks.cu", "runtime.cu", "noalloc.cu", "serve.cu", "sorted_grid.cu"]
-HEADERS = ["device.cuh", "kernels.h"]
+HEADERS = ["device.cuh", "cull.cuh", "kernels.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -23,6 +23,7 @@
 #include <atomic>
 #include <cstdint>
 
+#include "cull.cuh"
 #include "device.cuh"
 #include "kernels.h"
 
@@ -151,7 +152,7 @@ __global__ void __launch_bounds__(256) brick_split_kernel(BrickArgs a)
 {
     __shared__ unsigned s_start[257];
     __shared__ unsigned s_tmp[8];
-    __shared__ unsigned s_base, s_ebase;
+    __shared__ unsigned s_base, s_ebase, s_wbase;
     const unsigned tid = threadIdx.x, b0 = blockIdx.x * 256u, b = b0 + tid;
     if (b <= a.nbricks) s_start[tid] = brick_start(a, b);
     if (tid == 255u && b + 1u <= a.nbricks) s_start[256] = brick_start(a, b + 1u);
@@ -191,7 +192,11 @@ __global__ void __launch_bounds__(256) brick_split_kernel(BrickArgs a)
     unsigned total, etotal;
     const unsigned ex = block_excl_sum<256>(k, s_tmp, &total);
     const unsigned eex = block_excl_sum<256>(ok && m == 0u ? 1u : 0u, s_tmp, &etotal);
+    const unsigned words = a.masks && ok ? (m + 31u) / 32u : 0u;
+    unsigned wex = 0u, wtotal = 0u;
+    if (a.masks) wex = block_excl_sum<256>(words, s_tmp, &wtotal);
     if (tid == 0u) {
+        s_wbase = wtotal ? atomicAdd(&a.ctl->tickets[2], wtotal) : 0u;
         s_base = total ? atomicAdd(&a.ctl->tickets[3], total) : 0u;
         s_ebase = etotal ? atomicAdd(&a.ctl->tickets[6], etotal) : 0u;
     }
@@ -224,6 +229,16 @@ __global__ void __launch_bounds__(256) brick_split_kernel(BrickArgs a)
                 it.slot = k > 1u ? slot + j : NO_SLOT;
                 if (k > 1u) a.slot_meta[slot + j] = make_uint2(slot, k);
                 a.items[p + j] = it;
+            }
+            if (a.masks) {
+                const unsigned w0 = s_wbase + wex;
+                if (w0 + words > a.max_words) {   // never: max_words bounds the words of all items
+                    atomicOr(&a.ctl->err, ERR_RANGE);
+                    for (unsigned j = 0; j < k; ++j) a.mask0[p + j] = 0u;
+                } else {
+                    for (unsigned j = 0; j < k; ++j) a.mask0[p + j] = w0 + j * (BRICK_CHUNK / 32);
+                    for (unsigned q = 0; q < words; ++q) a.word_item[w0 + q] = p + q / (BRICK_CHUNK / 32);
+                }
             }
         }
     }
@@ -275,9 +290,72 @@ __device__ __forceinline__ void count_words(const BrickArgs &a, const BrickItem 
     }
 }
 
-// A warp per item.  A brick in one item writes its cells' counts; a chunk
-// writes its own to its slot, and the last chunk of the brick to arrive turns
-// the slots into offsets inside each cell and writes the sums.
+// Writes an item's counts (lane l of group g has cell 32 g + l; one warp).  A
+// brick in one item writes its cells' counts; a chunk writes its own to its
+// slot, and the last chunk of the brick to arrive turns the slots into offsets
+// inside each cell and writes the sums.
+__device__ __forceinline__ void finish_counts(const BrickArgs &a, const BrickItem &it, const Dims &d,
+                                              unsigned (&cnt)[GROUPS])
+{
+    const unsigned lane = threadIdx.x & 31u;
+    if (it.slot != NO_SLOT) {
+        unsigned *sl = a.slots + (size_t)it.slot * BRICK_CELLS;
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) sl[32 * g + lane] = cnt[g];
+        const uint2 meta = a.slot_meta[it.slot];
+        __threadfence();
+        __syncwarp();
+        unsigned last = 0u;
+        if (lane == 0u) last = atomicAdd(a.arrive + meta.x, 1u) + 1u == meta.y;
+        if (!__shfl_sync(FULL, last, 0)) return;
+        __threadfence();
+        // every chunk of the brick is counted: offsets of the chunks inside each cell
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) cnt[g] = 0u;
+        for (unsigned j = 0; j < meta.y; ++j) {
+            unsigned *sj = a.slots + (size_t)(meta.x + j) * BRICK_CELLS;
+            unsigned v[GROUPS];
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) v[g] = __ldcg(sj + 32 * g + lane);
+#pragma unroll
+            for (int g = 0; g < GROUPS; ++g) {
+                sj[32 * g + lane] = cnt[g];
+                cnt[g] += v[g];
+            }
+        }
+    }
+    unsigned most = 0u;
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) most = max(most, cnt[g]);
+    const bool big = most >= BRICK_BIG;
+    if (d.nx == 8u && d.ny == 8u && d.nz == 8u && !big) {   // a whole cube: steps of 4 rows and of a layer
+        unsigned short *p = a.counts + (it.cell0 + (lane & 7u) + it.rx * (lane >> 3));
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g)
+            p[(size_t)(g & 1) * (4u * it.rx) + (size_t)(g >> 1) * it.rxy] = (unsigned short)cnt[g];
+        return;
+    }
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) {
+        const unsigned c = 32u * g + lane;
+        const unsigned x = c & ((1u << d.lx) - 1u), y = (c >> d.lx) & ((1u << d.ly) - 1u), z = c >> (d.lx + d.ly);
+        if (x < d.nx && y < d.ny && z < d.nz) {
+            const unsigned cell = it.cell0 + x + it.rx * y + it.rxy * z;
+            a.counts[cell] = (unsigned short)min(cnt[g], BRICK_BIG);
+            if (cnt[g] >= BRICK_BIG) {
+                const unsigned k = atomicAdd(&a.ctl->tickets[1], 1u);
+                if (k < a.max_big)
+                    a.big[k] = make_uint2(cell, cnt[g]);
+                else
+                    atomicOr(&a.ctl->err, ERR_RANGE);   // never: a cell of the list holds 65,535 pairs
+            }
+        }
+    }
+}
+
+// A warp per item.  CULLED: the kept masks of its words instead of the boxes,
+// and their sum in ctl->nkept.
+template <bool CULLED>
 __global__ void __launch_bounds__(32 * COUNT_WARPS, 8) brick_count_kernel(BrickArgs a)
 {
     const unsigned lane = threadIdx.x & 31u;
@@ -289,60 +367,209 @@ __global__ void __launch_bounds__(32 * COUNT_WARPS, 8) brick_count_kernel(BrickA
         unsigned cnt[GROUPS];
 #pragma unroll
         for (int g = 0; g < GROUPS; ++g) cnt[g] = 0u;
-        count_words(a, it, d, cnt);
-        if (it.slot != NO_SLOT) {
-            unsigned *sl = a.slots + (size_t)it.slot * BRICK_CELLS;
+        if (CULLED) {
+            if (it.count) {
+                const unsigned *in = a.masks + (size_t)__ldg(a.mask0 + i) * BRICK_CELLS + lane;
+                for (unsigned e = 0; e < it.count; e += 32u, in += BRICK_CELLS) {
 #pragma unroll
-            for (int g = 0; g < GROUPS; ++g) sl[32 * g + lane] = cnt[g];
-            const uint2 meta = a.slot_meta[it.slot];
-            __threadfence();
+                    for (int g = 0; g < GROUPS; ++g) cnt[g] += __popc(__ldg(in + 32 * g));
+                }
+                unsigned sum = 0u;
+#pragma unroll
+                for (int g = 0; g < GROUPS; ++g) sum += cnt[g];
+                sum = __reduce_add_sync(FULL, sum);
+                if (lane == 0u && sum) atomicAdd(&a.ctl->nkept, (unsigned long long)sum);
+            }
+        } else {
+            count_words(a, it, d, cnt);
+        }
+        finish_counts(a, it, d, cnt);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// cull: the entries that each cell keeps, and their counts (culled builds)
+// ---------------------------------------------------------------------------
+
+// The test of cull.cuh decides every pair exactly as the pair path does; what
+// changes is which pairs reach it, and that full warps run it.  A word of 32
+// entries per warp: a lane sets up its entry's triangle and looks through the
+// box inside the brick when that has at most CULL_OWN cells; the warp looks
+// through a larger one, two rows of the brick per lane.  A cell that holds a
+// vertex is kept at once; one whose centre lies further from the triangle's
+// plane than any cell that the normal's axis could keep is dropped after one
+// multiply-add (most cells of a large triangle's box); the others are listed,
+// and the test runs over the list, a pair per lane.
+//
+// That bound, T: the test drops a cell when the three projections p_k = n . w_k
+// all lie beyond R = S (1/2 + max|w| 2^-16 + 2^-10) on one side.  With n
+// the FP32 cross product of FP32 edges of length at most L per component, n . e
+// is not zero but below 16 u L^3 (u = 2^-24), and the rounding of a projection
+// below 4 u S W <= 24 u L^2 W for W >= max|w| over the brick; the plane's own
+// value here is off by no more.  T = S (1/2 + W 2^-16 + 2^-10) (1 + 2^-10) +
+// 2^-18 L^2 (L + W) exceeds R by the sum of these.
+constexpr int CULL_WARPS = 4;
+constexpr unsigned CULL_OWN = 16;
+constexpr unsigned CULL_LIST = 512;   // pairs listed for the test
+static_assert(CULL_LIST >= BRICK_CELLS && CULL_LIST >= 32 * CULL_OWN, "one step lists no more than fits");
+constexpr int CULL_TRI = 25;   // words per triangle in shared memory (24 and a pad)
+
+__global__ void __launch_bounds__(32 * CULL_WARPS, 7) brick_cull_kernel(BrickArgs a)
+{
+    __shared__ unsigned s_keep[CULL_WARPS][BRICK_CELLS];   // per cell: the word's kept entries; zero between words
+    __shared__ float s_tri[CULL_WARPS][32 * CULL_TRI];
+    __shared__ unsigned short s_list[CULL_WARPS][CULL_LIST];   // (entry's lane, cell) of pairs to test
+    const unsigned lane = threadIdx.x & 31u, w = threadIdx.x >> 5, below = lanemask_lt();
+    const unsigned nwords = min(ld_relaxed_u32(&a.ctl->tickets[2]), a.max_words);
+    const float lo[3] = {a.lo[0], a.lo[1], a.lo[2]}, scale[3] = {a.scale[0], a.scale[1], a.scale[2]};
+    const float resf[3] = {(float)a.res[0], (float)a.res[1], (float)a.res[2]};
+    const unsigned zero3[3] = {0u, 0u, 0u};
+    const unsigned last3[3] = {(unsigned)a.res[0] - 1u, (unsigned)a.res[1] - 1u, (unsigned)a.res[2] - 1u};
+    unsigned *keep = s_keep[w];
+    float *tris = s_tri[w];
+    unsigned short *list = s_list[w];
+    for (unsigned c = lane; c < BRICK_CELLS; c += 32u) keep[c] = 0u;
+    __syncwarp();
+    for (unsigned word = blockIdx.x * CULL_WARPS + w; word < nwords; word += gridDim.x * CULL_WARPS) {
+        const unsigned item = __ldg(a.word_item + word);
+        const BrickItem it = load_item(a.items + item);
+        const unsigned q = word - __ldg(a.mask0 + item);
+        if (32u * q >= it.count) continue;   // never with consistent lists
+        const Dims d = decode(it.dims);
+        const unsigned lxy = d.lx + d.ly, mskx = (1u << d.lx) - 1u, msky = (1u << d.ly) - 1u;
+        const unsigned bz = it.cell0 / it.rxy, by = (it.cell0 - bz * it.rxy) / it.rx, bx = it.cell0 - bz * it.rxy - by * it.rx;
+        const unsigned org[3] = {bx, by, bz};   // the brick's first cell
+        const Entry en = load_entry(a, it.first + 32u * q, it.count - 32u * q);
+        const unsigned info = entry_info(a, en);
+        const unsigned l0 = info & (BRICK_CELLS - 1u), l1 = (info >> BRICK_CELLS_LOG) & (BRICK_CELLS - 1u);
+        const unsigned nx = (l1 & mskx) - (l0 & mskx) + 1u, ny = ((l1 >> d.lx) & msky) - ((l0 >> d.lx) & msky) + 1u;
+        const unsigned vol = en.ok ? nx * ny * ((l1 >> lxy) - (l0 >> lxy) + 1u) : 0u;
+        GridTri t;
+        unsigned live = 0u;
+        float A = 0.0f, T = 0.0f;   // the plane's value at the centre of the brick's first cell, the bound
+        if (en.ok) {
+            grid_tri(a.verts, a.nverts, a.tris, entry_obj(a, en), lo, scale, resf, t, a.ctl);
+            live = live_axes(t);
+            float W = 0.0f, L = 0.0f;
+            const unsigned ext[3] = {mskx, msky, (1u << d.lz) - 1u};
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) {
+                const float c0 = (float)org[ax] + 0.5f, c1 = c0 + (float)ext[ax];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    W = fmaxf(W, fmaxf(fabsf(t.q[3 * k + ax] - c0), fabsf(t.q[3 * k + ax] - c1)));
+                    L = fmaxf(L, fabsf(t.e[3 * k + ax]));
+                }
+                A = fmaf(t.n[ax], t.q[ax] - c0, A);
+            }
+            const float S = fabsf(t.n[0]) + fabsf(t.n[1]) + fabsf(t.n[2]);
+            T = fmaf(S, (0.5f + 9.765625e-04f + W * 1.52587890625e-05f) * 1.0009765625f,
+                     3.814697265625e-06f * (L * L) * (L + W));
+            if (!(live & 1u)) T = __int_as_float(0x7f800000);   // the test skips the normal: no bound from it
+        }
+        if (en.ok) {
+            float *o = tris + lane * CULL_TRI;
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                o[k] = t.q[k];
+                o[9 + k] = t.e[k];
+            }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) o[18 + k] = t.n[k];
+            o[21] = A;
+            o[22] = T;
+            o[23] = __uint_as_float(live);
+        }
+        unsigned listed = 0u;
+        auto append = [&](bool cand, unsigned c, unsigned e) {   // the lanes with cand list (e, c)
+            const unsigned m = __ballot_sync(FULL, cand);
+            if (cand) list[listed + __popc(m & below)] = (unsigned short)((e << BRICK_CELLS_LOG) | c);
+            listed += __popc(m);
+        };
+        auto test = [&]() {
             __syncwarp();
-            unsigned last = 0u;
-            if (lane == 0u) last = atomicAdd(a.arrive + meta.x, 1u) + 1u == meta.y;
-            if (!__shfl_sync(FULL, last, 0)) continue;
-            __threadfence();
-            // every chunk of the brick is counted: offsets of the chunks inside each cell
+            for (unsigned k = lane; k < listed; k += 32u) {
+                const unsigned v = list[k], c = v & (BRICK_CELLS - 1u), e = v >> BRICK_CELLS_LOG;
+                const float *o = tris + e * CULL_TRI;
+                GridTri g;
 #pragma unroll
-            for (int g = 0; g < GROUPS; ++g) cnt[g] = 0u;
-            for (unsigned j = 0; j < meta.y; ++j) {
-                unsigned *sj = a.slots + (size_t)(meta.x + j) * BRICK_CELLS;
-                unsigned v[GROUPS];
+                for (int j = 0; j < 9; ++j) {
+                    g.q[j] = o[j];
+                    g.e[j] = o[9 + j];
+                }
 #pragma unroll
-                for (int g = 0; g < GROUPS; ++g) v[g] = __ldcg(sj + 32 * g + lane);
+                for (int j = 0; j < 3; ++j) g.n[j] = o[18 + j];
+                if (!tri_cell_separated(g, __float_as_uint(o[23]), bx + (c & mskx), by + ((c >> d.lx) & msky),
+                                        bz + (c >> lxy)))
+                    atomicOr(&keep[c], 1u << e);
+            }
+            listed = 0u;
+            __syncwarp();
+        };
+        {
+            // boxes of few cells: the lane's own, cell by cell in box order
+            const bool own = vol <= CULL_OWN;
+            unsigned long long vc[3] = {0ull, 0ull, 0ull};
+            if (own && en.ok) {
 #pragma unroll
-                for (int g = 0; g < GROUPS; ++g) {
-                    sj[32 * g + lane] = cnt[g];
-                    cnt[g] += v[g];
+                for (int k = 0; k < 3; ++k) vc[k] = vertex_cell(t, k, zero3, last3);
+            }
+            unsigned c = l0, x = nx, y = ny;
+            const unsigned steps = __reduce_max_sync(FULL, own ? vol : 0u);
+            for (unsigned k = 0; k < steps; ++k) {
+                bool cand = own && k < vol;
+                if (cand) {
+                    const unsigned cx = c & mskx, cy = (c >> d.lx) & msky, cz = c >> lxy;
+                    const unsigned long long rc = (unsigned long long)(bx + cx) |
+                                                  ((unsigned long long)(by + cy) << 16) |
+                                                  ((unsigned long long)(bz + cz) << 32);
+                    if (rc == vc[0] || rc == vc[1] || rc == vc[2]) {
+                        atomicOr(&keep[c], 1u << lane);
+                        cand = false;
+                    } else {
+                        const float v =
+                            fmaf(-t.n[0], (float)cx, fmaf(-t.n[1], (float)cy, fmaf(-t.n[2], (float)cz, A)));
+                        cand = !(fabsf(v) > T);
+                    }
+                }
+                append(cand, c, lane);
+                ++c;
+                if (--x == 0u) {
+                    x = nx;
+                    c += (1u << d.lx) - nx;
+                    if (--y == 0u) {
+                        y = ny;
+                        c += (1u << lxy) - (ny << d.lx);
+                    }
                 }
             }
         }
-unsigned most = 0u;
-#pragma unroll
-        for (int g = 0; g < GROUPS; ++g) most = max(most, cnt[g]);
-        const bool big = most >= BRICK_BIG;
-        if (d.nx == 8u && d.ny == 8u && d.nz == 8u && !big) {   // a whole cube: steps of 4 rows and of a layer
-            unsigned short *p = a.counts + (it.cell0 + (lane & 7u) + it.rx * (lane >> 3));
-#pragma unroll
-            for (int g = 0; g < GROUPS; ++g)
-                p[(size_t)(g & 1) * (4u * it.rx) + (size_t)(g >> 1) * it.rxy] = (unsigned short)cnt[g];
-            continue;
+        __syncwarp();
+        for (unsigned large = __ballot_sync(FULL, vol > CULL_OWN); large; large &= large - 1u) {
+            const unsigned from = (unsigned)__ffs(large) - 1u;
+            const unsigned b0 = __shfl_sync(FULL, l0, from), bnx = __shfl_sync(FULL, nx, from),
+                           bny = __shfl_sync(FULL, ny, from), bv = __shfl_sync(FULL, vol, from);
+            const float *o = tris + from * CULL_TRI;
+            const float n0 = o[18], n1 = o[19], n2 = o[20], pA = o[21], pT = o[22];
+            const unsigned rx = 65535u / bnx + 1u, ry = 65535u / bny + 1u;   // exact quotients below 512
+            if (listed + bv > CULL_LIST) test();
+            for (unsigned k0 = 0; k0 < bv; k0 += 32u) {
+                const unsigned k = k0 + lane, u = (k * rx) >> 16, z = (u * ry) >> 16;
+                const unsigned c = b0 + (k - u * bnx) + ((u - z * bny) << d.lx) + (z << lxy);
+                const unsigned cx = c & mskx, cy = (c >> d.lx) & msky, cz = c >> lxy;
+                const float v = fmaf(-n0, (float)cx, fmaf(-n1, (float)cy, fmaf(-n2, (float)cz, pA)));
+                append(k < bv && !(fabsf(v) > pT), c & (BRICK_CELLS - 1u), from);
+            }
         }
+        if (listed) test();
+        __syncwarp();
+        unsigned *out = a.masks + (size_t)word * BRICK_CELLS;
 #pragma unroll
         for (int g = 0; g < GROUPS; ++g) {
-            const unsigned c = 32u * g + lane;
-            const unsigned x = c & ((1u << d.lx) - 1u), y = (c >> d.lx) & ((1u << d.ly) - 1u), z = c >> (d.lx + d.ly);
-            if (x < d.nx && y < d.ny && z < d.nz) {
-                const unsigned cell = it.cell0 + x + it.rx * y + it.rxy * z;
-                a.counts[cell] = (unsigned short)min(cnt[g], BRICK_BIG);
-                if (cnt[g] >= BRICK_BIG) {
-                    const unsigned k = atomicAdd(&a.ctl->tickets[1], 1u);
-                    if (k < a.max_big)
-                        a.big[k] = make_uint2(cell, cnt[g]);
-                    else
-                        atomicOr(&a.ctl->err, ERR_RANGE);   // never: a cell of the list holds 65,535 pairs
-                }
-            }
+            out[32 * g + lane] = keep[32 * g + lane];
+            keep[32 * g + lane] = 0u;
         }
+        __syncwarp();
     }
 }
 
@@ -598,19 +825,37 @@ constexpr int FILL_WARPS = 4;         // a warp per 128 cells of the brick
 static_assert(BRICK_CHUNK <= 1024, "10 bits of entry in a tag");
 static_assert(BRICK_CELLS == FILL_WARPS * 128, "four cells per lane");
 
+// The masks of a lane's four cells in word q: from the word's feature masks in
+// shared memory, or (culled builds) from the kept masks in device memory.
+struct BoxMasks {
+    const unsigned *mx, *my, *mz;
+    __device__ __forceinline__ uint4 operator()(unsigned q) const
+    {
+        const uint4 X = *reinterpret_cast<const uint4 *>(mx + MASK_PITCH * q);
+        const unsigned yz = my[MASK_PITCH * q] & mz[MASK_PITCH * q];
+        return make_uint4(X.x & yz, X.y & yz, X.z & yz, X.w & yz);
+    }
+};
+
+struct KeptMasks {
+    const unsigned *m;
+    __device__ __forceinline__ uint4 operator()(unsigned q) const
+    {
+        return __ldg(reinterpret_cast<const uint4 *>(m + (size_t)BRICK_CELLS * q));
+    }
+};
+
 // Stages the entries of words [q0, q1) that cover the lane's four cells, as
 // 16-bit tags: each cell's from its own position p on.  The four cells' lists
 // grow together, so finding an entry's bit is paid once for the cells it
 // covers.  A tag is `owner` over the entry; PER_CELL adds the cell of the four.
-template <bool PER_CELL>
-__device__ __forceinline__ void stage_entries(unsigned short *stage, const unsigned *mx, const unsigned *my,
-                                              const unsigned *mz, unsigned q0, unsigned q1, unsigned owner,
-                                              unsigned (&p)[4])
+template <bool PER_CELL, typename Masks>
+__device__ __forceinline__ void stage_entries(unsigned short *stage, const Masks &masks, unsigned q0, unsigned q1,
+                                              unsigned owner, unsigned (&p)[4])
 {
     for (unsigned q = q0; q < q1; ++q) {
-        const uint4 X = *reinterpret_cast<const uint4 *>(mx + MASK_PITCH * q);
-        const unsigned yz = my[MASK_PITCH * q] & mz[MASK_PITCH * q];
-        const unsigned m[4] = {X.x & yz, X.y & yz, X.z & yz, X.w & yz};
+        const uint4 M = masks(q);
+        const unsigned m[4] = {M.x, M.y, M.z, M.w};
         unsigned u = m[0] | m[1] | m[2] | m[3];
         const unsigned tag = owner | (q << 5);
         while (u) {
@@ -637,12 +882,12 @@ __device__ __forceinline__ void stage_entries(unsigned short *stage, const unsig
 // too).  128 cells go at once when their pairs fit the stage, else 32 cells at
 // a time, four lanes per four cells with a quarter of the entries each, and
 // where 32 cells do not fit either, in windows of entries.
-template <unsigned STAGE, int MIN_BLOCKS>
+template <unsigned STAGE, int MIN_BLOCKS, bool CULLED>
 __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel(BrickArgs a)
 {
     static_assert(STAGE >= 1024, "one word of 32 cells fits");
     constexpr unsigned W = FILL_WARPS;
-    __shared__ __align__(16) unsigned s_mask[BRICK_CHUNK / 32 * MASK_PITCH];   // [word of 32 entries][feature]
+    __shared__ __align__(16) unsigned s_mask[CULLED ? 4 : BRICK_CHUNK / 32 * MASK_PITCH];   // [word][feature]
     __shared__ unsigned s_obj[BRICK_CHUNK];
     __shared__ unsigned short s_stage[W][STAGE];
     __shared__ unsigned s_delta[W][32];                      // per cell: its refs' place less its staged place
@@ -684,11 +929,21 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
             const Entry cur = next;
             const unsigned en = 32u * (q + W);
             next = load_entry(a, it.first + en, en < it.count ? it.count - en : 0u);
-            s_mask[MASK_PITCH * q + lane] = transpose32(cur.ok ? feature_row(entry_info(a, cur), d) : 0u);
+            if (!CULLED) s_mask[MASK_PITCH * q + lane] = transpose32(cur.ok ? feature_row(entry_info(a, cur), d) : 0u);
             s_obj[32u * q + 31u - lane] = entry_obj(a, cur);
         }
         __syncthreads();
         const unsigned fy = 1u << d.lx, fz = fy + (1u << d.ly);
+        // the masks of four cells that start at local cell cc = (xx, yy, zz)
+        const unsigned *kept = CULLED ? a.masks + (size_t)__ldg(a.mask0 + i) * BRICK_CELLS : nullptr;
+        auto masks = [&](unsigned xx, unsigned yy, unsigned zz, unsigned cc) {
+            if constexpr (CULLED) {
+                return KeptMasks{kept + cc};
+            } else {
+                (void)cc;
+                return BoxMasks{s_mask + xx, s_mask + fy + yy, s_mask + ((fz + zz) & 31u)};
+            }
+        };
         const unsigned lsum = num[0] + num[1] + num[2] + num[3];
         const unsigned inc = warp_incl_sum(lsum);
         const unsigned total = __shfl_sync(FULL, inc, 31);
@@ -699,7 +954,7 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
             for (int k = 1; k < 4; ++k) p[k] = p[k - 1] + num[k - 1];
             const unsigned delta = dst[0] - p[0];   // the lane's cells follow one another in refs as in the stage
             if (lsum)
-                stage_entries<false>(stage, s_mask + x, s_mask + fy + y, s_mask + fz + z, 0u, nw, lane << 10, p);
+                stage_entries<false>(stage, masks(x, y, z, c0), 0u, nw, lane << 10, p);
             bad |= p[3] != inc;
             __syncwarp();
             for (unsigned p0 = 0; p0 < total; p0 += 32u) {
@@ -727,7 +982,7 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
             if (!__any_sync(FULL, live)) continue;
             const unsigned qx = __shfl_sync(FULL, x, from), qy = __shfl_sync(FULL, y, from),
                            qz = __shfl_sync(FULL, z, from);
-            const unsigned *mx = s_mask + qx, *my = s_mask + fy + qy, *mz = s_mask + ((fz + qz) & 31u);
+            const auto four = masks(qx, qy, qz, __shfl_sync(FULL, c0, from));
             unsigned win = nw;
             for (unsigned q0 = 0; q0 < nw;) {
                 unsigned nq = min(win, nw - q0), qa, qb, k[4], pre[4], sum[4], base, cnt;
@@ -737,12 +992,11 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
                     k[0] = k[1] = k[2] = k[3] = 0u;
                     if (live) {
                         for (unsigned q = qa; q < qb; ++q) {
-                            const uint4 X = *reinterpret_cast<const uint4 *>(mx + MASK_PITCH * q);
-                            const unsigned yz = my[MASK_PITCH * q] & mz[MASK_PITCH * q];
-                            k[0] += __popc(X.x & yz);
-                            k[1] += __popc(X.y & yz);
-                            k[2] += __popc(X.z & yz);
-                            k[3] += __popc(X.w & yz);
+                            const uint4 M = four(q);
+                            k[0] += __popc(M.x);
+                            k[1] += __popc(M.y);
+                            k[2] += __popc(M.z);
+                            k[3] += __popc(M.w);
                         }
                     }
                     // each cell's entries of the lower quarters, its sum, and the cells before
@@ -777,7 +1031,7 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
                     base += sum[j];
                     to[j] += sum[j];
                 }
-                if (live) stage_entries<true>(stage, mx, my, mz, qa, qb, quad << 12, p);
+                if (live) stage_entries<true>(stage, four, qa, qb, quad << 12, p);
                 __syncwarp();
                 for (unsigned p0 = lane; p0 < cnt; p0 += 32u) {
                     const unsigned v = stage[p0];
@@ -824,7 +1078,11 @@ cudaError_t launch_brick_split(const BrickArgs &a, cudaStream_t s)
 cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s)
 {
     const unsigned blocks = (a.max_items + COUNT_WARPS - 1u) / COUNT_WARPS, cap = (unsigned)nsm * 64u;
-    brick_count_kernel<<<blocks < cap ? blocks : cap, 32 * COUNT_WARPS, 0, s>>>(a);
+    const unsigned grid = blocks < cap ? blocks : cap;
+    if (a.masks)
+        brick_count_kernel<true><<<grid, 32 * COUNT_WARPS, 0, s>>>(a);
+    else
+        brick_count_kernel<false><<<grid, 32 * COUNT_WARPS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -848,10 +1106,26 @@ constexpr double DENSE_PAIRS_PER_CELL = 4.0;
 cudaError_t launch_brick_fill(const BrickArgs &a, int nsm, cudaStream_t s)
 {
     const unsigned cap = (unsigned)nsm * 64u, grid = a.max_items < cap ? a.max_items : cap;
-    if ((double)a.nrefs > DENSE_PAIRS_PER_CELL * (double)a.ncells_out)
-        brick_fill_kernel<2560, 8><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+    if (a.masks)
+        brick_fill_kernel<1024, 10, true><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+    else if ((double)a.nrefs > DENSE_PAIRS_PER_CELL * (double)a.ncells_out)
+        brick_fill_kernel<2560, 8, false><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
     else
-        brick_fill_kernel<1024, 10><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+        brick_fill_kernel<1024, 10, false><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+unsigned brick_max_words(unsigned nbricks, unsigned count)
+{
+    // every item rounds its last word up
+    const unsigned long long n = (unsigned long long)count / 32u + brick_max_items(nbricks < count ? nbricks : count, count);
+    return n > 0xFFFFFFFEull ? 0xFFFFFFFEu : (unsigned)n;
+}
+
+cudaError_t launch_brick_cull(const BrickArgs &a, int nsm, cudaStream_t s)
+{
+    const unsigned blocks = (a.max_words + CULL_WARPS - 1u) / CULL_WARPS, cap = (unsigned)nsm * 64u;
+    brick_cull_kernel<<<blocks < cap ? blocks : cap, 32 * CULL_WARPS, 0, s>>>(a);
     return cudaGetLastError();
 }
 

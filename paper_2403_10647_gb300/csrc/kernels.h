@@ -342,7 +342,17 @@ struct BrickArgs {
     unsigned long long *status;     // [cell_scan_tiles] look-back words, zeroed, or tile sums
     unsigned *refs;
     unsigned nrefs;
-    Ctl *ctl;                       // tickets [1], [3] .. [6] zero on entry
+    Ctl *ctl;                       // tickets [1] .. [6] zero on entry
+    // culled builds (single mesh): the mesh, and the entries that each cell keeps
+    const float *verts;
+    long long nverts;
+    const int *tris;
+    float lo[3], scale[3];
+    unsigned *masks;                // [max_words][BRICK_CELLS]: a word of 32 entries' mask per cell, entry k
+                                    // at bit 31 - k
+    unsigned *mask0;                // [max_items]: an item's first word
+    unsigned *word_item;            // [max_words]: a word's item
+    unsigned max_words;             // tickets [2] counts the words
 };
 constexpr unsigned BRICK_BIG = 65535u;
 
@@ -353,6 +363,9 @@ cudaError_t launch_brick_split(const BrickArgs &a, cudaStream_t s);
 cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s);
 cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s);
 cudaError_t launch_brick_fill(const BrickArgs &a, int nsm, cudaStream_t s);
+// Culled builds: the cull before count.
+unsigned brick_max_words(unsigned nbricks, unsigned count);
+cudaError_t launch_brick_cull(const BrickArgs &a, int nsm, cudaStream_t s);
 
 unsigned long long extract_blocks(unsigned long long count, unsigned long long ncells);
 cudaError_t launch_extract_split(const ExtractArgs &a, cudaStream_t s);

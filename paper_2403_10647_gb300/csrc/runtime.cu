@@ -103,6 +103,7 @@ struct grid_ctx {
     Scratch b_desc, b_base, b_state, b_pairbase, b_cellsoff, b_G;   // batched builds
     Scratch b_seg;                  // batched builds sorted in segments: the segments' tables
     Scratch items, slots, slot_meta, counts;   // brick builds: work items, chunk counts, cell counts
+    Scratch masks, mask0;        // culled brick builds: kept entries per word and cell, each item's first word
     Scratch bstart, btile_obj;   // brick builds: each object's first entry, each entry tile's object
     Scratch pairs_C, pairs_O;    // object-order pairs of the unfused pair_gen modes and of culling
     void *h_stage = nullptr;     // pinned host tables of batched builds (grow-only)
@@ -697,11 +698,10 @@ int bits_of(unsigned long long v)   // bits of the largest of v values, at least
 unsigned long long axis_bricks(int res, unsigned l) { return ((unsigned long long)res + (1u << l) - 1) >> l; }
 
 // May a context build by bricks (radix passes over (brick, object) entries)?
-// Every explicit choice of pair generation or sort end, and culling, keeps the
-// pair path.
+// Every explicit choice of pair generation or sort end keeps the pair path.
 bool may_use_bricks(const grid_ctx *c)
 {
-    return c->local_bits == 0 && c->pair_gen == GRID_PAIRS_FUSED && !c->cull;
+    return c->local_bits == 0 && c->pair_gen == GRID_PAIRS_FUSED;
 }
 
 // Does it, for a scene of NO pairs in `entries` brick entries?  Where an entry
@@ -718,11 +718,12 @@ bool bricks_pay(int64_t NO, int64_t entries)
     return NO >= BRICK_MIN_PAIRS && NO >= BRICK_MIN_PAIRS_PER_ENTRY * entries;
 }
 
-// RadixSort .. ExclusiveSum by bricks, after the count: entries generated and
-// sorted by brick, then split, count, scan and fill (bricks.cu) write cells
-// (ncells_out words) and refs.  la: shapes, meshes and packing are set.
-int place_bricks(grid_ctx *c, gg::BrickArgs a, const gg::BrickGen &bg, unsigned entries, int64_t nobj,
-                 const unsigned *tile_obj, OutAlloc *out)
+// The first half of a brick build, after the count: entries generated and sorted
+// by brick, then listed as work items; the scratch of the rest.  a: shapes,
+// meshes, packing, ncells_out and nrefs (or a bound of it) are set, its buffers
+// are filled in.
+int sort_bricks(grid_ctx *c, gg::BrickArgs &a, const gg::BrickGen &bg, unsigned entries, int64_t nobj,
+                const unsigned *tile_obj)
 {
     const SortCfg sc = sort_cfg(a.kb, c->rbits_max);
     GG_TRY(ensure(c, c->keys_sorted, (size_t)entries * sizeof(unsigned)));
@@ -751,22 +752,64 @@ int place_bricks(grid_ctx *c, gg::BrickArgs a, const gg::BrickGen &bg, unsigned 
     GG_TRY(ensure(c, c->k2status, tiles * 8));   // the count's look-back words are done with
     a.status = (unsigned long long *)c->k2status.ptr;
     GG_CUDA(cudaMemsetAsync(a.status, 0, tiles * 8, c->stream));
-    {
-        KernelScope ks(c, K_BSPLIT, 4.0 * a.nbricks);
-        GG_CUDA(gg::launch_brick_split(a, c->stream));
-    }
-    {
-        KernelScope ks(c, K_BCOUNT, 8.0 * entries + 2.0 * a.ncells_out);
-        GG_CUDA(gg::launch_brick_count(a, c->nsm, c->stream));
-    }
+    KernelScope ks(c, K_BSPLIT, 4.0 * a.nbricks);
+    GG_CUDA(gg::launch_brick_split(a, c->stream));
+    return GRID_OK;
+}
+
+// The second half, after every cell's objects are counted: cells (a.G) and
+// refs.
+int fill_bricks(grid_ctx *c, const gg::BrickArgs &a, OutAlloc *out)
+{
     {
         KernelScope ks(c, K_CSCAN, 6.0 * a.ncells_out);
         GG_CUDA(gg::launch_cell_scan(a, c->stream));
     }
     if (out) GG_TRY(out->cells_ready(c, a.G, a.ncells_out));
-    KernelScope ks(c, K_LOCAL, 8.0 * entries + 4.0 * a.ncells_out + 4.0 * a.nrefs);
+    KernelScope ks(c, K_LOCAL, 8.0 * a.count + 4.0 * a.ncells_out + 4.0 * a.nrefs);
     GG_CUDA(gg::launch_brick_fill(a, c->nsm, c->stream));
     return GRID_OK;
+}
+
+// RadixSort .. ExclusiveSum by bricks, after the count (bricks.cu).
+int place_bricks(grid_ctx *c, gg::BrickArgs a, const gg::BrickGen &bg, unsigned entries, int64_t nobj,
+                 const unsigned *tile_obj, OutAlloc *out)
+{
+    GG_TRY(sort_bricks(c, a, bg, entries, nobj, tile_obj));
+    {
+        KernelScope ks(c, K_BCOUNT, 8.0 * entries + 2.0 * a.ncells_out);
+        GG_CUDA(gg::launch_brick_count(a, c->nsm, c->stream));
+    }
+    return fill_bricks(c, a, out);
+}
+
+// The same for a culled build: the pairs that the triangle / cell test keeps
+// are counted (*nkept, synchronises), then the outputs are allocated.
+int place_bricks_culled(grid_ctx *c, gg::BrickArgs a, const gg::BrickGen &bg, unsigned entries, int64_t nobj,
+                        const unsigned *tile_obj, OutAlloc *out, int64_t *nkept)
+{
+    a.max_words = gg::brick_max_words(a.nbricks, entries);
+    GG_TRY(ensure(c, c->masks, (size_t)a.max_words * gg::BRICK_CELLS * sizeof(unsigned)));
+    GG_TRY(ensure(c, c->mask0, ((size_t)gg::brick_max_items(a.nbricks, entries) + a.max_words) * sizeof(unsigned)));
+    a.masks = (unsigned *)c->masks.ptr;
+    a.word_item = (unsigned *)c->mask0.ptr;
+    a.mask0 = a.word_item + a.max_words;
+    GG_TRY(sort_bricks(c, a, bg, entries, nobj, tile_obj));
+    {
+        KernelScope ks(c, K_CULL, 8.0 * entries + 48.0 * nobj + 4.0 * gg::BRICK_CELLS / 32 * entries);
+        GG_CUDA(gg::launch_brick_cull(a, c->nsm, c->stream));
+    }
+    {
+        KernelScope ks(c, K_BCOUNT, 4.0 * gg::BRICK_CELLS / 32 * entries + 2.0 * a.ncells_out);
+        GG_CUDA(gg::launch_brick_count(a, c->nsm, c->stream));
+    }
+    GG_TRY(read_ctl(c));
+    GG_TRY(ctl_error(c->h_ctl->err));
+    *nkept = (int64_t)c->h_ctl->nkept;
+    GG_TRY(out->alloc(c, a.ncells_out, *nkept, &a.G, &a.refs));
+    a.nrefs = (unsigned)*nkept;
+    GG_TRY(fill_bricks(c, a, out));
+    return out->refs_ready(c, a.refs, *nkept);
 }
 
 // Culling emit over the box placement's NO pairs: the kept pairs, compacted
@@ -952,7 +995,6 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
         bg.kb = bits_of(nbx * nby * nbz);
         bg.ob = bits_of((unsigned long long)n);
         if (bricks_pay(NO, entries) && gg::brick_packs(bg.kb, bg.ob)) {
-            GG_TRY(out.alloc(c, I.ncells + 1, NO, &cells, &refs));
             const unsigned ntiles = pair_tiles(entries);
             const bool tiles_done = ca.btile_obj && (size_t)ntiles + 1 <= ca.btile_cap &&
                                     !(c->h_ctl->err & gg::ERR_BTILE_REDO);
@@ -970,12 +1012,22 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
             ba.shape = bg.shape;
             ba.nbx = bg.nbx;
             ba.nby = bg.nby;
-            ba.G = cells;
             ba.ncells_out = I.ncells + 1;
-            ba.refs = refs;
             ba.nrefs = (unsigned)NO;
-            GG_TRY(place_bricks(c, ba, bg, entries, n, tile_obj, &out));
-            GG_TRY(out.refs_ready(c, refs, NO));
+            if (c->cull) {
+                ba.verts = verts;
+                ba.nverts = nverts;
+                ba.tris = tris;
+                for (int a = 0; a < 3; ++a) {
+                    ba.lo[a] = I.lo[a];
+                    ba.scale[a] = I.scale[a];
+                }
+                GG_TRY(place_bricks_culled(c, ba, bg, entries, n, tile_obj, &out, &I.nrefs));
+            } else {
+                GG_TRY(out.alloc(c, I.ncells + 1, NO, &ba.G, &ba.refs));
+                GG_TRY(place_bricks(c, ba, bg, entries, n, tile_obj, &out));
+                GG_TRY(out.refs_ready(c, ba.refs, NO));
+            }
             GG_TRY(read_ctl(c));
             GG_TRY(ctl_error(c->h_ctl->err));
             if (info) *info = I;
@@ -1280,7 +1332,7 @@ void grid_ctx_destroy(grid_ctx *c)
                           &c->vals_sorted, &c->bstarts, &c->bgroups,
                           &c->vals[0], &c->intra, &c->gpref, &c->gstatus, &c->in_verts, &c->in_tris,
                           &c->out_cells, &c->out_refs, &c->b_desc, &c->b_base, &c->b_state, &c->b_pairbase,
-                          &c->b_cellsoff, &c->b_G, &c->b_seg, &c->items, &c->slots, &c->slot_meta, &c->counts,
+                          &c->b_cellsoff, &c->b_G, &c->b_seg, &c->items, &c->slots, &c->slot_meta, &c->counts, &c->masks, &c->mask0,
                           &c->bstart, &c->btile_obj, &c->pairs_C, &c->pairs_O, &c->cstatus};
         for (Scratch *s : all) release(c, *s);
         if (c->stream) cudaStreamSynchronize(c->stream);

@@ -68,6 +68,22 @@ def test_brick_builds_match_oracle(name):
         c.close()
 
 
+@pytest.mark.parametrize("name", ["cube", "thin_z", "flat_z", "flat_x", "line_z", "few_cells", "soup"])
+def test_culled_brick_builds_match_oracle(name):
+    """Culled brick builds: the same test decides, whichever pairs reach it
+    (boxes of a lane and of the warp, planes that miss most of a box)."""
+    import paper_2403_10647_gb300 as pg
+    s = scenes.nonhomogeneous_soup(70_000, seed=31, extent=30.0) if name == "soup" else SCENES[name]()
+    o = oracle.build_grid(s.verts, s.tris, s.lam, cull=True)
+    c = pg.Context(0, cull=True)
+    try:
+        c.profile(True)
+        assert_grid_equal(c.build(dev(s.verts, torch.float32), dev(s.tris, torch.int32), s.lam), o, name)
+        assert "cell_scan" in c.kernel_stats()
+    finally:
+        c.close()
+
+
 def test_brick_batch_matches_oracle():
     import paper_2403_10647_gb300 as pg
     empty = scenes.Scene("empty", np.zeros((0, 3), np.float32), np.zeros((0, 3), np.int32), 4.0)
