@@ -271,13 +271,61 @@ __device__ __forceinline__ void gen_bricks(const ObjRec *__restrict__ recs, cons
 }
 
 // ---------------------------------------------------------------------------
+// a1 on the device: grid metadata M from the bounds (one thread)
+// ---------------------------------------------------------------------------
+
+__device__ void device_plan(Ctl *ctl, long long n, float lambda)
+{
+    float lo[3], e[3];
+    int res[3] = {1, 1, 1};
+    float scale[3] = {0.0f, 0.0f, 0.0f};
+    const bool ok = __ldcg(&ctl->err) == 0u && n > 0;
+    int d = 0;
+    double vol = 1.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        // the bounds as the host reads them: a zero bound is +0.0
+        lo[a] = ok ? __fadd_rn(ordered_to_float(~__ldcg(&ctl->lo_inv[a])), 0.0f) : 0.0f;
+        const float hi = ok ? __fadd_rn(ordered_to_float(__ldcg(&ctl->hi_ord[a])), 0.0f) : 0.0f;
+        e[a] = __fsub_rn(hi, lo[a]);
+        if (ok && e[a] > 0.0f) {
+            ++d;
+            vol = __dmul_rn(vol, (double)e[a]);
+        }
+    }
+    if (d > 0) {
+        const double q = __ddiv_rn(__dmul_rn((double)lambda, (double)n), vol);
+        const double k = d == 3 ? cbrt(q) : (d == 2 ? __dsqrt_rn(q) : q);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (!(e[a] > 0.0f)) continue;
+            double r = ceil(__dmul_rn((double)e[a], k));
+            if (!(r >= 1.0)) r = 1.0;
+            if (r > 65535.0) r = 65535.0;
+            res[a] = (int)r;
+            scale[a] = __fdiv_rn((float)res[a], e[a]);
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        ctl->plan_lo[a] = lo[a];
+        ctl->plan_scale[a] = scale[a];
+        ctl->plan_res[a] = res[a];
+    }
+}
+
+// ---------------------------------------------------------------------------
 // a0: boxes + scene bounds
 // ---------------------------------------------------------------------------
 
 __global__ void __launch_bounds__(256) bounds_kernel(const float *__restrict__ verts, long long nverts,
                                                      const int *__restrict__ tris, long long n,
-                                                     Ctl *ctl)
+                                                     Ctl *ctl, BoundsExtra x)
 {
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < x.zero[k].words; i += gridDim.x * blockDim.x)
+            x.zero[k].p[i] = 0u;
     float lo[3] = {__int_as_float(0x7f800000), __int_as_float(0x7f800000), __int_as_float(0x7f800000)};
     float hi[3] = {-lo[0], -lo[1], -lo[2]};
     unsigned err = 0;
@@ -335,6 +383,16 @@ __global__ void __launch_bounds__(256) bounds_kernel(const float *__restrict__ v
         atomicMax(&ctl->hi_ord[threadIdx.x], s_hi[threadIdx.x]);
     }
     if (threadIdx.x == 0 && s_err) atomicOr(&ctl->err, s_err);
+    if (!x.plan) return;
+    // the last block to finish plans: one launch less, but a fence and an atomic per block
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&ctl->bounds_done, 1u) + 1u == gridDim.x) {
+            __threadfence();
+            device_plan(ctl, n, x.lambda);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -520,51 +578,12 @@ __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(Cou
     }
     if (tile_redo) atomicOr(&a.ctl->err, ERR_TILE_REDO);
     if (BRICKS && btile_redo) atomicOr(&a.ctl->err, ERR_BTILE_REDO);
+    publish_ctl(a.ctl, a.host, &a.ctl->count_done);
 }
-
-// ---------------------------------------------------------------------------
-// a1 on the device: grid metadata M from the bounds
-// ---------------------------------------------------------------------------
 
 __global__ void plan_kernel(Ctl *ctl, long long n, float lambda)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    float lo[3], e[3];
-    int res[3] = {1, 1, 1};
-    float scale[3] = {0.0f, 0.0f, 0.0f};
-    const bool ok = ctl->err == 0u && n > 0;
-    int d = 0;
-    double vol = 1.0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        // the bounds as the host reads them: a zero bound is +0.0
-        lo[a] = ok ? __fadd_rn(ordered_to_float(~ctl->lo_inv[a]), 0.0f) : 0.0f;
-        const float hi = ok ? __fadd_rn(ordered_to_float(ctl->hi_ord[a]), 0.0f) : 0.0f;
-        e[a] = __fsub_rn(hi, lo[a]);
-        if (ok && e[a] > 0.0f) {
-            ++d;
-            vol = __dmul_rn(vol, (double)e[a]);
-        }
-    }
-    if (d > 0) {
-        const double q = __ddiv_rn(__dmul_rn((double)lambda, (double)n), vol);
-        const double k = d == 3 ? cbrt(q) : (d == 2 ? __dsqrt_rn(q) : q);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (!(e[a] > 0.0f)) continue;
-            double r = ceil(__dmul_rn((double)e[a], k));
-            if (!(r >= 1.0)) r = 1.0;
-            if (r > 65535.0) r = 65535.0;
-            res[a] = (int)r;
-            scale[a] = __fdiv_rn((float)res[a], e[a]);
-        }
-    }
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        ctl->plan_lo[a] = lo[a];
-        ctl->plan_scale[a] = scale[a];
-        ctl->plan_res[a] = res[a];
-    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) device_plan(ctl, n, lambda);
 }
 
 cudaError_t launch_plan(Ctl *ctl, long long n, float lambda, cudaStream_t s)
@@ -1379,6 +1398,7 @@ __global__ void __launch_bounds__(BLOCK) extract_kernel(ExtractArgs a)
     // below would wrap)
     if (i1 < i0 || i1 - i0 > d1 - d0) {
         if (threadIdx.x == 0) atomicOr(&a.ctl->err, ERR_RANGE);
+        publish_ctl(a.ctl, a.host, &a.ctl->place_done);
         return;
     }
     // every key before i0 is below c0 and every key from i1 on is at least
@@ -1437,6 +1457,7 @@ __global__ void __launch_bounds__(BLOCK) extract_kernel(ExtractArgs a)
         // lanes are a few cells apart, so a warp's stores share sectors
         a.G[(unsigned long long)c0 + k] = (unsigned)i0 + pos;
     }
+    publish_ctl(a.ctl, a.host, &a.ctl->place_done);
 }
 
 // ---------------------------------------------------------------------------
@@ -1810,6 +1831,7 @@ __global__ void __launch_bounds__(BLOCK, LOCAL_MIN_BLOCKS) local_sort_kernel(Loc
     }
     if (bad) atomicOr(&a.ctl->err, ERR_RANGE);
     }
+    publish_ctl(a.ctl, a.host, &a.ctl->place_done);
 }
 
 // ---------------------------------------------------------------------------
@@ -1976,13 +1998,18 @@ __global__ void __launch_bounds__(256) rebase_recs_kernel(ObjRec *__restrict__ r
 // ---------------------------------------------------------------------------
 
 cudaError_t launch_bounds(const float *verts, long long nverts, const int *tris, long long n, Ctl *ctl,
-                          int nsm, cudaStream_t s)
+                          int nsm, cudaStream_t s, BoundsExtra *x, bool *planned)
 {
+    if (planned) *planned = false;
     if (n <= 0) return cudaSuccess;
     long long blocks = (n + 255) / 256;
     const long long cap = (long long)nsm * 8;
     if (blocks > cap) blocks = cap;
-    bounds_kernel<<<(unsigned)blocks, 256, 0, s>>>(verts, nverts, tris, n, ctl);
+    BoundsExtra e{};
+    if (x) e = *x;
+    if (blocks > 4 * nsm) e.plan = false;   // beyond, the blocks' atomics cost more than the launch
+    if (planned) *planned = e.plan;
+    bounds_kernel<<<(unsigned)blocks, 256, 0, s>>>(verts, nverts, tris, n, ctl, e);
     return cudaGetLastError();
 }
 

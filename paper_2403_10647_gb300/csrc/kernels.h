@@ -100,6 +100,7 @@ struct CountArgs {
     unsigned *tile_obj;             // single mesh, optional: [tile_cap] the first object of every
     unsigned tile_cap;              // PAIR_TILE-pair tile and, after the last tile, n - 1 (tile_search's
                                     // result), or ERR_TILE_REDO when it did not fit
+    Ctl *host;                      // optional: publish_ctl's mirror
     bool bricks;                    // count and scan the brick entries too:
     unsigned *bstart;               // [n] out: the exclusive prefix sum of the entries
     unsigned *btile_obj;            // as tile_obj for tiles of PAIR_TILE entries, or ERR_BTILE_REDO
@@ -193,6 +194,7 @@ struct ExtractArgs {
     unsigned *G;                    // [ncells + 1]
     unsigned *splits;               // [extract_blocks + 1] merge-path splits (scratch)
     Ctl *ctl;
+    Ctl *host;                      // optional: publish_ctl's mirror
 };
 
 // Per-request vertex jitter of the serving loop: dst[e] = src[e] + s * n(e)
@@ -213,8 +215,20 @@ struct JitterDesc {
 cudaError_t launch_jitter(const JitterDesc &one, const JitterDesc *d, const long long *ebase, int nm,
                           long long total, cudaStream_t s);
 
+// Words that the bounds kernel zeroes for the kernels after it, so that a small
+// build needs no memsets, and the plan (launch_plan's) in its last block when
+// there are few blocks; *planned tells whether that is so.
+struct ZeroRange {
+    unsigned *p;
+    unsigned words;
+};
+struct BoundsExtra {
+    ZeroRange zero[3];
+    bool plan;
+    float lambda;
+};
 cudaError_t launch_bounds(const float *verts, long long nverts, const int *tris, long long n, Ctl *ctl,
-                          int nsm, cudaStream_t s);
+                          int nsm, cudaStream_t s, BoundsExtra *x = nullptr, bool *planned = nullptr);
 // Batched: per-mesh bounds into bstate[m * 6 + (lo_inv x, y, z, hi x, y, z)].
 cudaError_t launch_bounds_batched(const MeshTab &mt, long long ntot, unsigned *bstate, Ctl *ctl, cudaStream_t s);
 // Batched: out[q] = G[q - m] - pair_base[m] for q in mesh m's slice
@@ -292,6 +306,7 @@ struct LocalArgs {
     unsigned *refs;                 // [count] out: object ids in cell order
     unsigned *G;                    // [ncells + 1] out
     Ctl *ctl;                       // tickets[2] counts the groups (zero on entry)
+    Ctl *host;                      // optional: publish_ctl's mirror
 };
 
 // starts[b] = number of keys whose key >> lbits is below b, b = 0 .. nbuckets;

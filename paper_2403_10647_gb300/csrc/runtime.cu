@@ -92,7 +92,11 @@ struct grid_ctx {
     int64_t fallbacks = 0;       // hybrid placements redone by radix passes over every key bit
     int64_t plan_redos = 0;      // builds whose device M differed from the host's
 
-    Ctl *d_ctl = nullptr;        // device control block
+    Ctl *d_ctl = nullptr;        // device control block: one of the two ctls
+    Ctl *ctls[2] = {nullptr, nullptr};
+    bool ctl_zero[2] = {false, false};   // zeroed by an earlier build, not used since
+    unsigned gzero_words = 0;    // words of gstatus that this build's bounds kernel zeroed
+    bool published = false;      // the last kernel enqueued writes h_ctl itself
     Ctl *h_ctl = nullptr;        // pinned host mirror
     unsigned *d_dbase = nullptr; // [MAX_PASSES][MAX_RADIX]
 
@@ -279,15 +283,45 @@ float bound_hi(unsigned hi_ord) { return gg::ordered_to_float(hi_ord) + 0.0f; }
 
 int read_ctl(grid_ctx *c)
 {
-    GG_CUDA(cudaMemcpyAsync(c->h_ctl, c->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
+    const bool published = c->published;
+    c->published = false;
+    if (!published)
+        GG_CUDA(cudaMemcpyAsync(c->h_ctl, c->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
     GG_CUDA(cudaStreamSynchronize(c->stream));
     return GRID_OK;
 }
 
 int reset_ctl(grid_ctx *c)
 {
+    c->gzero_words = 0;
+    c->published = false;
+    c->ctl_zero[c->d_ctl == c->ctls[1]] = false;
     GG_CUDA(cudaMemsetAsync(c->d_ctl, 0, sizeof(Ctl), c->stream));
     return GRID_OK;
+}
+
+// A zeroed control block for a build: the one that the last build zeroed
+// (builds end with the stream synchronised) if it did.
+int next_ctl(grid_ctx *c)
+{
+    const int k = c->d_ctl == c->ctls[1] ? 0 : 1;
+    c->d_ctl = c->ctls[k];
+    if (!c->ctl_zero[k]) return reset_ctl(c);
+    c->ctl_zero[k] = false;
+    c->gzero_words = 0;
+    c->published = false;
+    return GRID_OK;
+}
+
+// Builds below these sizes end their host waits with publish_ctl instead of a
+// copy (its atomic per block is nothing then, a copy's 4 us are).
+constexpr int64_t PUBLISH_MAX_OBJECTS = 1ll << 20, PUBLISH_MAX_PAIRS = 1ll << 22;
+
+// The mirror for a kernel that precedes a host wait, or null for a copy.
+Ctl *publish(grid_ctx *c, bool small)
+{
+    c->published = small;
+    return small ? c->h_ctl : nullptr;
 }
 
 // ---- grid metadata M -------------------------------------------------------
@@ -405,9 +439,10 @@ int sort_pairs(grid_ctx *c, const SortCfg &sc, unsigned count, bool gen, const O
     // every pass gets its own zeroed look-back words: one clear for the sort
     const size_t status_words = (size_t)ngroups * R;
     GG_TRY(ensure(c, c->gstatus, (size_t)std::max(sc.passes, 1) * status_words * sizeof(unsigned)));
-    if (sc.passes > 0)
+    if (sc.passes > 0 && c->gzero_words < sc.passes * status_words)
         GG_CUDA(cudaMemsetAsync(c->gstatus.ptr, 0, (size_t)sc.passes * status_words * sizeof(unsigned),
                                 c->stream));
+    c->gzero_words = 0;   // used up
     if (sc.passes > 1 || store) {
         GG_TRY(ensure(c, c->keys[0], elem));
         GG_TRY(ensure(c, c->vals[0], elem));
@@ -497,7 +532,8 @@ bool valid_lambda(float lambda) { return std::isfinite(lambda) && lambda > 0.0f;
 
 // RunLengthEncode + NonEmptyCells + ExclusiveSum: merge-path splits, then the
 // per-block merge of sorted keys against cell ids.
-int extract_ranges(grid_ctx *c, const unsigned *keys, int64_t count, int64_t ncells, unsigned *cells)
+int extract_ranges(grid_ctx *c, const unsigned *keys, int64_t count, int64_t ncells, unsigned *cells,
+                   bool last = false)
 {
     const unsigned long long nb = gg::extract_blocks((unsigned long long)count, (unsigned long long)ncells);
     GG_TRY(ensure(c, c->splits, (size_t)(nb + 1) * sizeof(unsigned)));
@@ -512,6 +548,7 @@ int extract_ranges(grid_ctx *c, const unsigned *keys, int64_t count, int64_t nce
         KernelScope ks(c, K_SPLIT, 4.0 * (nb + 1));
         GG_CUDA(gg::launch_extract_split(xa, c->stream));
     }
+    if (last) xa.host = publish(c, count <= PUBLISH_MAX_PAIRS);   // the build's last kernel
     KernelScope ks(c, K_EXTRACT, 4.0 * count + 4.0 * (ncells + 1));
     GG_CUDA(gg::launch_extract(xa, c->stream));
     return GRID_OK;
@@ -561,10 +598,10 @@ int choose_local_bits(const grid_ctx *c, int key_bits, int64_t count, int64_t nc
 // radix passes order the pairs by the key bits from L up (the first pass
 // generating them when gen is set, else reading keys_in / vals_in), then
 // one block per bucket of 2^L cells sorts its pairs by cell in shared memory
-// and writes the bucket's part of cells (G) and refs.
+// and writes the bucket's part of cells (G) and refs.  last: the host waits next.
 int sort_place(grid_ctx *c, int key_bits, int64_t ncells, unsigned count, bool gen, const ObjRec *recs,
                int64_t nobj, const unsigned *tile_obj, unsigned res_x, unsigned res_y, const gg::MeshTab &mt,
-               const unsigned *keys_in, const unsigned *vals_in, unsigned *refs, unsigned *cells)
+               const unsigned *keys_in, const unsigned *vals_in, unsigned *refs, unsigned *cells, bool last)
 {
     const int L = choose_local_bits(c, key_bits, count, ncells);
     const SortCfg sc = sort_cfg(key_bits, c->rbits_max, L, GG_FIRST_EXTRA);
@@ -613,8 +650,8 @@ int sort_place(grid_ctx *c, int key_bits, int64_t ncells, unsigned count, bool g
     la.groups = (unsigned *)c->bgroups.ptr;
     la.refs = refs;
     la.G = cells;
-    la.ctl = c->d_ctl;
-    GG_CUDA(cudaMemsetAsync(&c->d_ctl->tickets[2], 0, sizeof(unsigned), c->stream));
+    la.ctl = c->d_ctl;   // its tickets[2] is zero: a build places its pairs this way once
+    if (last) la.host = publish(c, count <= PUBLISH_MAX_PAIRS);
     {
         KernelScope ks(c, K_BSPLIT, 4.0 * (la.nbuckets + 1));
         GG_CUDA(gg::launch_bucket_split(la, c->stream));
@@ -901,18 +938,32 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
     }
     // a0: boxes + bounds, a1 on the device, a2 + a3 with the device's M: one
     // host synchronisation for bounds, M and NO together
-    GG_TRY(reset_ctl(c));
-    {
-        KernelScope ks(c, K_BOUNDS, 48.0 * n);
-        GG_CUDA(gg::launch_bounds(verts, nverts, tris, n, c->d_ctl, c->nsm, c->stream));
-    }
-    {
-        KernelScope ks(c, K_PLAN, 0.0);
-        GG_CUDA(gg::launch_plan(c->d_ctl, n, lambda, c->stream));
-    }
+    GG_TRY(next_ctl(c));
     const int64_t ctiles = (n + gg::COUNT_TILE - 1) / gg::COUNT_TILE;
     GG_TRY(ensure(c, c->recs, (size_t)n * sizeof(ObjRec)));
     GG_TRY(ensure(c, c->k2status, (size_t)ctiles * 8));
+    // zeroed on the way: the count's look-back words, the sort's as far as they
+    // are kept from earlier builds and few, the next build's control block
+    const int other = c->d_ctl == c->ctls[1] ? 0 : 1;
+    const int64_t bounds_blocks = std::min<int64_t>((n + 255) / 256, 8 * c->nsm);
+    const unsigned gzero = (unsigned)std::min<int64_t>(
+        {(int64_t)(c->gstatus.bytes / sizeof(unsigned)), 2048 * bounds_blocks, 1ll << 20});
+    gg::BoundsExtra bx{};
+    bx.zero[0] = gg::ZeroRange{(unsigned *)c->k2status.ptr, (unsigned)(2 * ctiles)};
+    bx.zero[1] = gg::ZeroRange{(unsigned *)c->gstatus.ptr, gzero};
+    bx.zero[2] = gg::ZeroRange{(unsigned *)c->ctls[other], (unsigned)(sizeof(Ctl) / sizeof(unsigned))};
+    bx.plan = true;
+    bx.lambda = lambda;
+    bool planned = false;
+    {
+        KernelScope ks(c, K_BOUNDS, 48.0 * n);
+        GG_CUDA(gg::launch_bounds(verts, nverts, tris, n, c->d_ctl, c->nsm, c->stream, &bx, &planned));
+    }
+    c->gzero_words = gzero;
+    if (!planned) {
+        KernelScope ks(c, K_PLAN, 0.0);
+        GG_CUDA(gg::launch_plan(c->d_ctl, n, lambda, c->stream));
+    }
     gg::CountArgs ca{};
     ca.verts = verts;
     ca.nverts = nverts;
@@ -934,13 +985,14 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
     ca.tile_obj = (unsigned *)c->tile_obj.ptr;
     ca.tile_cap = (unsigned)std::min<size_t>(c->tile_obj.bytes / sizeof(unsigned), 0xFFFFFFFFull);
     auto count_scan = [&]() -> int {
-        GG_CUDA(cudaMemsetAsync(c->k2status.ptr, 0, (size_t)ctiles * 8, c->stream));
+        ca.host = publish(c, n <= PUBLISH_MAX_OBJECTS);
         KernelScope ks(c, K_COUNT, 64.0 * n);
         GG_CUDA(gg::launch_count_scan(ca, c->stream));
         return GRID_OK;
     };
     GG_TRY(count_scan());
     GG_TRY(read_ctl(c));
+    c->ctl_zero[other] = true;
     if (c->h_ctl->err & (gg::ERR_BADINDEX | gg::ERR_NONFINITE)) return GRID_EINVAL;
     float lo[3], hi[3];
     for (int a = 0; a < 3; ++a) {
@@ -973,6 +1025,8 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
         GG_CUDA(cudaMemsetAsync(&c->d_ctl->err, 0, sizeof(unsigned), c->stream));
         GG_CUDA(cudaMemsetAsync(&c->d_ctl->tickets[0], 0, sizeof(unsigned), c->stream));
         GG_CUDA(cudaMemsetAsync(&c->d_ctl->npairs, 0, sizeof(c->d_ctl->npairs), c->stream));
+        GG_CUDA(cudaMemsetAsync(&c->d_ctl->count_done, 0, sizeof(unsigned), c->stream));
+        GG_CUDA(cudaMemsetAsync(c->k2status.ptr, 0, (size_t)ctiles * 8, c->stream));
         GG_TRY(count_scan());
         GG_TRY(read_ctl(c));
     }
@@ -1047,7 +1101,7 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
         GG_TRY(out.alloc(c, I.ncells + 1, NK, &cells, &refs));
         if (NK > 0 && use_hybrid(c, NK, I.ncells)) {
             GG_TRY(sort_place(c, I.key_bits, I.ncells, (unsigned)NK, false, nullptr, 0, nullptr, 0, 0, gg::MeshTab{},
-                              C, O, refs, cells));
+                              C, O, refs, cells, true));
             GG_TRY(out.refs_ready(c, refs, NK));
             GG_TRY(read_ctl(c));
             GG_TRY(ctl_error(c->h_ctl->err));
@@ -1074,7 +1128,7 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
                 keys = (const unsigned *)c->keys_sorted.ptr;
             }
             GG_TRY(out.refs_ready(c, refs, kc));
-            GG_TRY(extract_ranges(c, keys, kc, I.ncells, cells));
+            GG_TRY(extract_ranges(c, keys, kc, I.ncells, cells, true));
         } else {
             GG_CUDA(cudaMemsetAsync(cells, 0, (size_t)(I.ncells + 1) * sizeof(unsigned), c->stream));
         }
@@ -1112,7 +1166,7 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
             }
             const unsigned rx = (unsigned)I.res[0], ry = (unsigned)I.res[1];
             GG_TRY(sort_place(c, I.key_bits, I.ncells, count, !in_memory, recs, n, tile_obj, rx, ry, gg::MeshTab{}, C,
-                              O, refs, cells));
+                              O, refs, cells, true));
             GG_TRY(out.refs_ready(c, refs, count));
             GG_TRY(read_ctl(c));
             GG_TRY(ctl_error(c->h_ctl->err));
@@ -1148,7 +1202,7 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
                               gg::MeshTab{}, nullptr, nullptr, keys_sorted, refs));
         }
         GG_TRY(out.refs_ready(c, refs, count));
-        GG_TRY(extract_ranges(c, keys_sorted, count, I.ncells, cells));
+        GG_TRY(extract_ranges(c, keys_sorted, count, I.ncells, cells, true));
     } else {
         GG_CUDA(cudaMemsetAsync(cells, 0, (size_t)(I.ncells + 1) * sizeof(unsigned), c->stream));
     }
@@ -1304,12 +1358,13 @@ int grid_ctx_create(int device, const grid_opts *opts, grid_ctx **out)
         if ((rc = cuda_err(cudaMemPoolCreate(&c->pool, &props)))) break;
         uint64_t thr = UINT64_MAX;
         if ((rc = cuda_err(cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &thr)))) break;
-        const size_t small = sizeof(Ctl) + sizeof(unsigned) * gg::MAX_PASSES * gg::MAX_RADIX;
+        const size_t small = 2 * sizeof(Ctl) + sizeof(unsigned) * gg::MAX_PASSES * gg::MAX_RADIX;
         void *p = nullptr;
         if ((rc = cuda_err(cudaMalloc(&p, small)))) break;
         if ((rc = cuda_err(cudaMemset(p, 0, small)))) break;
-        c->d_ctl = (Ctl *)p;
-        c->d_dbase = (unsigned *)((char *)p + sizeof(Ctl));
+        c->ctls[0] = c->d_ctl = (Ctl *)p;
+        c->ctls[1] = c->ctls[0] + 1;
+        c->d_dbase = (unsigned *)(c->ctls[0] + 2);
         if ((rc = cuda_err(cudaMallocHost(&p, sizeof(Ctl))))) break;
         c->h_ctl = (Ctl *)p;
         std::memset(c->h_ctl, 0, sizeof(Ctl));
@@ -1339,7 +1394,7 @@ void grid_ctx_destroy(grid_ctx *c)
         resolve_timings(c);
         for (cudaEvent_t e : c->free_events) cudaEventDestroy(e);
         c->free_events.clear();
-        if (c->d_ctl) cudaFree(c->d_ctl);
+        if (c->ctls[0]) cudaFree(c->ctls[0]);
         if (c->h_ctl) cudaFreeHost(c->h_ctl);
         if (c->h_stage) cudaFreeHost(c->h_stage);
         if (c->pool) cudaMemPoolDestroy(c->pool);
@@ -2084,7 +2139,7 @@ int grid_build_batched(grid_ctx *c, const grid_mesh *meshes, int32_t nmeshes, gr
             const SortCfg sc = sort_cfg(key_bits, c->rbits_max);
             if (use_hybrid(c, count, ncells_all)) {
                 GG_TRY(sort_place(c, key_bits, ncells_all, count, true, recs, ntot, tile_obj, 0, 0, mt, nullptr, nullptr,
-                                  (unsigned *)pr, G));
+                                  (unsigned *)pr, G, false));
             } else if (sc.passes == 0) {
                 gg::EmitArgs ea{};
                 ea.recs = recs;
