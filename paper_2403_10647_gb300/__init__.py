@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes
 import dataclasses
+import struct
 
 import numpy as np
 
@@ -18,6 +19,14 @@ from . import _lib
 from ._lib import GridError, GridInfo, GridBuf, GridOpts, GridServeOpts, GridServeStats, check
 
 __all__ = ["Context", "Server", "Info", "Grid", "BatchedGrids", "plan", "GridError"]
+
+
+# grid_info in one read: a ctypes array per field costs more than a small build's launches
+_INFO = struct.Struct("=9f4i4x3q")
+assert _INFO.size == ctypes.sizeof(GridInfo)
+# grid_mesh, filled for all meshes of a batch at once
+_MESH = np.dtype([("verts", "u8"), ("nverts", "i8"), ("tris", "u8"), ("n", "i8"), ("lam", "f4"), ("reserved", "i4")])
+assert _MESH.itemsize == ctypes.sizeof(_lib.GridMesh)
 
 
 @dataclasses.dataclass
@@ -33,8 +42,8 @@ class Info:
 
     @classmethod
     def from_c(cls, i: GridInfo) -> "Info":
-        return cls(tuple(i.lo), tuple(i.hi), tuple(i.scale), tuple(i.res), int(i.key_bits),
-                   int(i.ncells), int(i.nrefs), int(i.n))
+        v = _INFO.unpack(bytes(i))
+        return cls(v[0:3], v[3:6], v[6:9], v[9:12], v[12], v[13], v[14], v[15])
 
     def to_c(self) -> GridInfo:
         c = GridInfo()
@@ -134,6 +143,9 @@ class Context:
         import torch
         self._torch = torch
         self.device = torch.device("cuda", device)
+        # the handle of the current stream, without a Stream object where torch gives it so
+        self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+            lambda index: torch.cuda.current_stream(index).cuda_stream)
         self._lib = _lib.load()
         opts = GridOpts()
         opts.radix_bits = int(radix_bits)
@@ -161,9 +173,8 @@ class Context:
         # torch's default stream is the legacy default stream (handle 0); it is
         # bound as cudaStreamLegacy, as NULL would select the context's own
         # non-blocking stream, which does not order with torch's work
-        s = self._torch.cuda.current_stream(self.device)
-        h = s.cuda_stream or _lib.CUDA_STREAM_LEGACY
-        check(self._lib.grid_ctx_set_stream(self._h, ctypes.c_void_p(h)), "grid_ctx_set_stream")
+        h = self._raw_stream(self.device.index) or _lib.CUDA_STREAM_LEGACY
+        check(self._lib.grid_ctx_set_stream(self._h, h), "grid_ctx_set_stream")
 
     def _dev(self, t, dtype, cols=None):
         torch = self._torch
@@ -212,15 +223,11 @@ class Context:
 
     def _mesh_array(self, meshes):
         torch = self._torch
-        keep = []
-        arr = (_lib.GridMesh * len(meshes))()
-        for m, (verts, tris, lam) in enumerate(meshes):
-            v = self._dev(verts, torch.float32, 3)
-            t = self._dev(tris, torch.int32, 3)
-            keep += [v, t]
-            arr[m].verts, arr[m].nverts = v.data_ptr(), v.shape[0]
-            arr[m].tris, arr[m].n, arr[m].lam = t.data_ptr(), t.shape[0], float(lam)
-        return arr, keep
+        f32, i32, dev = torch.float32, torch.int32, self._dev
+        keep = [(dev(verts, f32, 3), dev(tris, i32, 3), float(lam)) for verts, tris, lam in meshes]
+        rows = np.array([(v.data_ptr(), v.size(0), t.data_ptr(), t.size(0), lam, 0) for v, t, lam in keep], dtype=_MESH)
+        arr = (_lib.GridMesh * len(keep)).from_buffer(rows) if len(keep) else (_lib.GridMesh * 0)()
+        return arr, (keep, rows)
 
     def autotune_batched(self, meshes, reps: int = 3) -> dict:
         """Times the batch `meshes` ((verts, tris, lam) each) built as one with
