@@ -32,7 +32,7 @@ namespace gg {
 #define GG_COUNT_TILE 2048
 #endif
 #ifndef GG_COUNT_MIN_BLOCKS
-#define GG_COUNT_MIN_BLOCKS 6
+#define GG_COUNT_MIN_BLOCKS 5
 #endif
 constexpr int COUNT_BLOCK = GG_COUNT_BLOCK;
 constexpr int COUNT_TILE = GG_COUNT_TILE;
