@@ -919,6 +919,7 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
                 if (x + k < d.nx) {
                     dst[k] = it.base + g[k];
                     num[k] = g[k + 1] - g[k];
+                    bad |= num[k] > a.nrefs || dst[k] > a.nrefs - num[k];
                     // the cell's other chunks come first; this one's share is counted below
                     if (it.slot != NO_SLOT) dst[k] += __ldg(a.slots + (size_t)it.slot * BRICK_CELLS + c0 + k);
                 }
@@ -944,6 +945,8 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
                 return BoxMasks{s_mask + xx, s_mask + fy + yy, s_mask + ((fz + zz) & 31u)};
             }
         };
+        // a cells array that points outside refs (never with consistent lists): nothing is written
+        if (__any_sync(FULL, bad)) continue;
         const unsigned lsum = num[0] + num[1] + num[2] + num[3];
         const unsigned inc = warp_incl_sum(lsum);
         const unsigned total = __shfl_sync(FULL, inc, 31);
@@ -955,18 +958,14 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
             const unsigned delta = dst[0] - p[0];   // the lane's cells follow one another in refs as in the stage
             if (lsum)
                 stage_entries<false>(stage, masks(x, y, z, c0), 0u, nw, lane << 10, p);
-            bad |= p[3] != inc;
             __syncwarp();
-            for (unsigned p0 = 0; p0 < total; p0 += 32u) {
-                const unsigned q = p0 + lane;
-                const unsigned v = q < total ? stage[q] : 0u;
-                const unsigned r = q + __shfl_sync(FULL, delta, v >> 10);
-                if (q < total) {
-                    if (r < a.nrefs)
-                        __stcs(a.refs + r, s_obj[v & 1023u]);
-                    else
-                        bad = true;
-                }
+            for (unsigned p0 = 0; p0 < total; p0 += 64u) {   // two refs per lane in flight
+                const unsigned q0 = p0 + lane, q1 = q0 + 32u;
+                const unsigned v0 = q0 < total ? stage[q0] : 0u, v1 = q1 < total ? stage[q1] : 0u;
+                const unsigned r0 = q0 + __shfl_sync(FULL, delta, v0 >> 10), r1 = q1 + __shfl_sync(FULL, delta, v1 >> 10);
+                const unsigned o0 = s_obj[v0 & 1023u], o1 = s_obj[v1 & 1023u];
+                if (q0 < total) __stcs(a.refs + r0, o0);
+                if (q1 < total) __stcs(a.refs + r1, o1);
             }
             __syncwarp();
             continue;
@@ -1033,13 +1032,17 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
                 }
                 if (live) stage_entries<true>(stage, four, qa, qb, quad << 12, p);
                 __syncwarp();
-                for (unsigned p0 = lane; p0 < cnt; p0 += 32u) {
+                unsigned p0 = lane;
+                for (; p0 + 32u < cnt; p0 += 64u) {   // two refs per lane in flight
+                    const unsigned v0 = stage[p0], v1 = stage[p0 + 32u];
+                    const unsigned r0 = p0 + sdelta[v0 >> 10], r1 = p0 + 32u + sdelta[v1 >> 10];
+                    const unsigned o0 = s_obj[v0 & 1023u], o1 = s_obj[v1 & 1023u];
+                    __stcs(a.refs + r0, o0);
+                    __stcs(a.refs + r1, o1);
+                }
+                if (p0 < cnt) {
                     const unsigned v = stage[p0];
-                    const unsigned r = p0 + sdelta[v >> 10];
-                    if (r < a.nrefs)
-                        __stcs(a.refs + r, s_obj[v & 1023u]);
-                    else
-                        bad = true;
+                    __stcs(a.refs + (p0 + sdelta[v >> 10]), s_obj[v & 1023u]);
                 }
                 __syncwarp();
                 q0 += nq;
