@@ -873,6 +873,30 @@ __device__ __forceinline__ void stage_entries(unsigned short *stage, const Masks
     }
 }
 
+// The same, staging the entries' objects.
+template <typename Masks>
+__device__ __forceinline__ void stage_objects(unsigned *stage, const unsigned *s_obj, const Masks &masks, unsigned q0,
+                                              unsigned q1, unsigned (&p)[4])
+{
+    for (unsigned q = q0; q < q1; ++q) {
+        const uint4 M = masks(q);
+        const unsigned m[4] = {M.x, M.y, M.z, M.w};
+        unsigned u = m[0] | m[1] | m[2] | m[3];
+        while (u) {
+            const unsigned b = __clz(u), t = 0x80000000u >> b;
+            u &= ~t;
+            const unsigned v = s_obj[32u * q + b];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (m[i] & t) {
+                    stage[p[i]] = v;
+                    ++p[i];
+                }
+            }
+        }
+    }
+}
+
 // A block per item, a warp per 128 cells, four neighbours in x per lane.  Of
 // every four rows each warp takes another one, skewed from layer to layer: a
 // surface that follows a plane of the brick keeps all warps busy.  The
@@ -882,14 +906,21 @@ __device__ __forceinline__ void stage_entries(unsigned short *stage, const Masks
 // too).  128 cells go at once when their pairs fit the stage, else 32 cells at
 // a time, four lanes per four cells with a quarter of the entries each, and
 // where 32 cells do not fit either, in windows of entries.
-template <unsigned STAGE, int MIN_BLOCKS, bool CULLED>
+//
+// DENSE: where 128 cells do not fit the stage (and no four cells overflow it on
+// their own) the objects themselves are staged, for 8, 4, 2 or 1 lanes' cells
+// at a time, the other lanes sharing their entries; four cells' refs are one
+// run then, copied by whole warps without a tag, a lookup of its place and
+// one of its object per ref.  Shared memory bounds the fill there (91% of its
+// rate with tags): 1.47 -> 1.26 ms on the soup of 7.3M triangles, 1.0e9 refs.
+template <unsigned STAGE, int MIN_BLOCKS, bool CULLED, bool DENSE>
 __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel(BrickArgs a)
 {
     static_assert(STAGE >= 1024, "one word of 32 cells fits");
     constexpr unsigned W = FILL_WARPS;
     __shared__ __align__(16) unsigned s_mask[CULLED ? 4 : BRICK_CHUNK / 32 * MASK_PITCH];   // [word][feature]
     __shared__ unsigned s_obj[BRICK_CHUNK];
-    __shared__ unsigned short s_stage[W][STAGE];
+    __shared__ __align__(16) unsigned short s_stage[W][STAGE];
     __shared__ unsigned s_delta[W][32];                      // per cell: its refs' place less its staged place
     const unsigned lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
     const unsigned nitems = min(ld_relaxed_u32(&a.ctl->tickets[3]), a.max_items);
@@ -968,6 +999,51 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
                 if (q1 < total) __stcs(a.refs + r1, o1);
             }
             __syncwarp();
+            continue;
+        }
+        if (DENSE && it.slot == NO_SLOT && !__any_sync(FULL, lsum > STAGE / 2u)) {
+            unsigned *ostage = reinterpret_cast<unsigned *>(stage);
+            for (unsigned l0 = 0; l0 < 32u;) {   // the cells of lanes l0 .. l0 + nl - 1
+                const unsigned before = l0 ? __shfl_sync(FULL, inc, l0 - 1u) : 0u;
+                unsigned nl = l0 + 8u <= 32u ? 8u : l0 + 4u <= 32u ? 4u : l0 + 2u <= 32u ? 2u : 1u;
+                while (__shfl_sync(FULL, inc, l0 + nl - 1u) - before > STAGE / 2u) nl >>= 1;
+                const unsigned q = lane & (nl - 1u), from = l0 + q, subs = 32u / nl, sub = lane / nl;
+                const unsigned len = __shfl_sync(FULL, lsum, from), at = __shfl_sync(FULL, inc, from) - len - before;
+                const unsigned to = __shfl_sync(FULL, dst[0], from);
+                const auto four = masks(__shfl_sync(FULL, x, from), __shfl_sync(FULL, y, from), __shfl_sync(FULL, z, from),
+                                        __shfl_sync(FULL, c0, from));
+                const unsigned n0 = __shfl_sync(FULL, num[0], from), n1 = __shfl_sync(FULL, num[1], from),
+                               n2 = __shfl_sync(FULL, num[2], from);
+                const unsigned qa = nw * sub / subs, qb = nw * (sub + 1u) / subs;
+                unsigned k[4] = {0u, 0u, 0u, 0u}, p[4] = {at, at + n0, at + n0 + n1, at + n0 + n1 + n2};
+                if (len) {
+                    for (unsigned qq = qa; qq < qb; ++qq) {
+                        const uint4 M = four(qq);
+                        k[0] += __popc(M.x);
+                        k[1] += __popc(M.y);
+                        k[2] += __popc(M.z);
+                        k[3] += __popc(M.w);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {   // behind the entries of the lanes that share the cells before this one
+                    unsigned v = k[j];
+                    for (unsigned o = nl; o < 32u; o <<= 1) {
+                        const unsigned t = __shfl_up_sync(FULL, v, o);
+                        if (lane >= o) v += t;
+                    }
+                    p[j] += v - k[j];
+                }
+                if (len) stage_objects(ostage, s_obj, four, qa, qb, p);
+                __syncwarp();
+                for (unsigned i4 = 0; i4 < nl; ++i4) {
+                    const unsigned n = __shfl_sync(FULL, len, i4), src = __shfl_sync(FULL, at, i4);
+                    unsigned *out = a.refs + __shfl_sync(FULL, to, i4);
+                    for (unsigned r = lane; r < n; r += 32u) __stcs(out + r, ostage[src + r]);
+                }
+                __syncwarp();
+                l0 += nl;
+            }
             continue;
         }
         const unsigned quad = lane & 7u, sub = lane >> 3;
@@ -1102,19 +1178,19 @@ cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s)
 }
 
 // Beyond 4 pairs per cell the larger stage wins, below the more resident blocks:
-// 165 against 225 us on the soup of 1M triangles (19 pairs per cell), 812
-// against 724 us on the building of 10M (2.4).
+// 132 against 150 us on the soup of 1M triangles (19 pairs per cell), 812
+// against 724 us on the building of 10M (2.4; an earlier form of the kernel).
 constexpr double DENSE_PAIRS_PER_CELL = 4.0;
 
 cudaError_t launch_brick_fill(const BrickArgs &a, int nsm, cudaStream_t s)
 {
     const unsigned cap = (unsigned)nsm * 64u, grid = a.max_items < cap ? a.max_items : cap;
     if (a.masks)
-        brick_fill_kernel<1024, 10, true><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+        brick_fill_kernel<1024, 10, true, false><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
     else if ((double)a.nrefs > DENSE_PAIRS_PER_CELL * (double)a.ncells_out)
-        brick_fill_kernel<2560, 8, false><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+        brick_fill_kernel<3072, 6, false, true><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
     else
-        brick_fill_kernel<1024, 10, false><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+        brick_fill_kernel<1024, 10, false, true><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
