@@ -1184,7 +1184,9 @@ constexpr double DENSE_PAIRS_PER_CELL = 4.0;
 
 cudaError_t launch_brick_fill(const BrickArgs &a, int nsm, cudaStream_t s)
 {
-    const unsigned cap = (unsigned)nsm * 64u, grid = a.max_items < cap ? a.max_items : cap;
+    // many more blocks than fit, so that bricks of many entries even out: 638 us at the 10M building, 656 with 64
+    // per SM, 667 with a block per item
+    const unsigned cap = (unsigned)nsm * 256u, grid = a.max_items < cap ? a.max_items : cap;
     if (a.masks)
         brick_fill_kernel<1024, 10, true, false><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
     else if ((double)a.nrefs > DENSE_PAIRS_PER_CELL * (double)a.ncells_out)
