@@ -106,9 +106,9 @@ struct grid_ctx {
     Scratch in_verts, in_tris, out_cells, out_refs;  // host-buffer builds
     Scratch b_desc, b_base, b_state, b_pairbase, b_cellsoff, b_G;   // batched builds
     Scratch b_seg;                  // batched builds sorted in segments: the segments' tables
-    Scratch items, slots, slot_meta, counts;   // brick builds: work items, chunk counts, cell counts
+    Scratch bricks;              // brick builds, one block: work items, chunk counts, cell counts
     Scratch masks, mask0;        // culled brick builds: kept entries per word and cell, each item's first word
-    Scratch bstart, btile_obj;   // brick builds: each object's first entry, each entry tile's object
+    Scratch btile_obj;           // brick builds: each entry tile's first object
     Scratch pairs_C, pairs_O;    // object-order pairs of the unfused pair_gen modes and of culling
     void *h_stage = nullptr;     // pinned host tables of batched builds (grow-only)
     size_t h_stage_bytes = 0;
@@ -475,7 +475,7 @@ int sort_pairs(grid_ctx *c, const SortCfg &sc, unsigned count, bool gen, const O
         u.res_y = res_y;
         if (bg) {
             u.bg = *bg;
-            u.bstart = (const unsigned *)c->bstart.ptr;
+            u.bstart = (const unsigned *)(recs + nobj);   // behind the records (brick_recs)
         }
         u.gen_keys = first ? gk : nullptr;
         u.gen_vals = first ? gv : nullptr;
@@ -741,6 +741,15 @@ bool may_use_bricks(const grid_ctx *c)
     return c->local_bits == 0 && c->pair_gen == GRID_PAIRS_FUSED;
 }
 
+// The records of n objects and, for a count with brick entries, each object's
+// first entry behind them: one block.
+int brick_recs(grid_ctx *c, int64_t n, bool bricks, unsigned **bstart)
+{
+    GG_TRY(ensure(c, c->recs, (size_t)n * (sizeof(ObjRec) + (bricks ? sizeof(unsigned) : 0))));
+    *bstart = bricks ? (unsigned *)((ObjRec *)c->recs.ptr + n) : nullptr;
+    return GRID_OK;
+}
+
 // Does it, for a scene of NO pairs in `entries` brick entries?  Where an entry
 // stands for few pairs, or there are few pairs in all, the bricks' extra steps
 // (split, count, scan: three launches) cost more than the shorter sort saves.
@@ -773,18 +782,23 @@ int sort_bricks(grid_ctx *c, gg::BrickArgs &a, const gg::BrickGen &bg, unsigned 
                       (unsigned *)c->keys_sorted.ptr, (unsigned *)c->vals_sorted.ptr, false, &bg));
     a.max_items = gg::brick_max_items(a.nbricks, entries);
     a.max_slots = gg::brick_max_slots(entries);
-    GG_TRY(ensure(c, c->items, (size_t)a.max_items * sizeof(gg::BrickItem)));
-    GG_TRY(ensure(c, c->slots, (size_t)a.max_slots * gg::BRICK_CELLS * sizeof(unsigned)));
-    GG_TRY(ensure(c, c->slot_meta, (size_t)a.max_slots * (sizeof(uint2) + sizeof(unsigned))));
-    a.items = (gg::BrickItem *)c->items.ptr;
-    a.slots = (unsigned *)c->slots.ptr;
-    a.slot_meta = (uint2 *)c->slot_meta.ptr;
-    a.arrive = (unsigned *)(a.slot_meta + a.max_slots);
     a.max_big = a.nrefs / gg::BRICK_BIG + 1u;
-    const size_t count_bytes = ((size_t)a.ncells_out * sizeof(unsigned short) + 255) & ~size_t(255);
-    GG_TRY(ensure(c, c->counts, count_bytes + (size_t)a.max_big * sizeof(uint2)));
-    a.counts = (unsigned short *)c->counts.ptr;
-    a.big = (uint2 *)((char *)c->counts.ptr + count_bytes);
+    const size_t sizes[6] = {(size_t)a.max_items * sizeof(gg::BrickItem),
+                             (size_t)a.max_slots * gg::BRICK_CELLS * sizeof(unsigned),
+                             (size_t)a.max_slots * sizeof(uint2),
+                             (size_t)a.max_slots * sizeof(unsigned),
+                             (size_t)a.ncells_out * sizeof(unsigned short),
+                             (size_t)a.max_big * sizeof(uint2)};
+    size_t at[7] = {0};
+    for (int k = 0; k < 6; ++k) at[k + 1] = at[k] + ((sizes[k] + 255) & ~size_t(255));
+    GG_TRY(ensure(c, c->bricks, at[6]));
+    char *base = (char *)c->bricks.ptr;
+    a.items = (gg::BrickItem *)base;
+    a.slots = (unsigned *)(base + at[1]);
+    a.slot_meta = (uint2 *)(base + at[2]);
+    a.arrive = (unsigned *)(base + at[3]);
+    a.counts = (unsigned short *)(base + at[4]);
+    a.big = (uint2 *)(base + at[5]);
     const size_t tiles = (size_t)gg::cell_scan_tiles(a.ncells_out);
     GG_TRY(ensure(c, c->k2status, tiles * 8));   // the count's look-back words are done with
     a.status = (unsigned long long *)c->k2status.ptr;
@@ -940,7 +954,8 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
     // host synchronisation for bounds, M and NO together
     GG_TRY(next_ctl(c));
     const int64_t ctiles = (n + gg::COUNT_TILE - 1) / gg::COUNT_TILE;
-    GG_TRY(ensure(c, c->recs, (size_t)n * sizeof(ObjRec)));
+    unsigned *bstart = nullptr;
+    GG_TRY(brick_recs(c, n, may_use_bricks(c), &bstart));
     GG_TRY(ensure(c, c->k2status, (size_t)ctiles * 8));
     // zeroed on the way: the count's look-back words, the sort's as far as they
     // are kept from earlier builds and few, the next build's control block
@@ -975,8 +990,7 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
     ca.device_plan = true;
     ca.bricks = may_use_bricks(c);
     if (ca.bricks) {
-        GG_TRY(ensure(c, c->bstart, (size_t)n * sizeof(unsigned)));
-        ca.bstart = (unsigned *)c->bstart.ptr;
+        ca.bstart = bstart;
         ca.btile_obj = (unsigned *)c->btile_obj.ptr;
         ca.btile_cap = (unsigned)std::min<size_t>(c->btile_obj.bytes / sizeof(unsigned), 0xFFFFFFFFull);
     }
@@ -1056,8 +1070,7 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
             unsigned *tile_obj = (unsigned *)c->btile_obj.ptr;
             if (!tiles_done) {
                 KernelScope ks(c, K_TILES, 4.0 * (ntiles + 1));
-                GG_CUDA(gg::launch_tile_search((const unsigned *)c->bstart.ptr, 1, n, gg::PAIR_TILE, ntiles, tile_obj,
-                                               c->stream));
+                GG_CUDA(gg::launch_tile_search(bstart, 1, n, gg::PAIR_TILE, ntiles, tile_obj, c->stream));
             }
             ba.nbricks = (unsigned)(nbx * nby * nbz);
             ba.kb = bg.kb;
@@ -1387,8 +1400,7 @@ void grid_ctx_destroy(grid_ctx *c)
                           &c->vals_sorted, &c->bstarts, &c->bgroups,
                           &c->vals[0], &c->intra, &c->gpref, &c->gstatus, &c->in_verts, &c->in_tris,
                           &c->out_cells, &c->out_refs, &c->b_desc, &c->b_base, &c->b_state, &c->b_pairbase,
-                          &c->b_cellsoff, &c->b_G, &c->b_seg, &c->items, &c->slots, &c->slot_meta, &c->counts, &c->masks, &c->mask0,
-                          &c->bstart, &c->btile_obj, &c->pairs_C, &c->pairs_O, &c->cstatus};
+                          &c->b_cellsoff, &c->b_G, &c->b_seg, &c->bricks, &c->masks, &c->mask0, &c->btile_obj, &c->pairs_C, &c->pairs_O, &c->cstatus};
         for (Scratch *s : all) release(c, *s);
         if (c->stream) cudaStreamSynchronize(c->stream);
         resolve_timings(c);
@@ -2035,10 +2047,10 @@ int grid_build_batched(grid_ctx *c, const grid_mesh *meshes, int32_t nmeshes, gr
 
     // a2 + a3 over all objects: one scan, so each mesh's pairs follow the last
     const int64_t ctiles = (ntot + gg::COUNT_TILE - 1) / gg::COUNT_TILE;
-    unsigned *pair_base_d = (unsigned *)c->b_pairbase.ptr;
+    unsigned *pair_base_d = (unsigned *)c->b_pairbase.ptr, *bstart = nullptr;
     GG_CUDA(cudaMemsetAsync(pair_base_d, 0, sizeof(unsigned) * nm, c->stream));
     if (ntot > 0) {
-        GG_TRY(ensure(c, c->recs, (size_t)ntot * sizeof(ObjRec)));
+        GG_TRY(brick_recs(c, ntot, may_brick, &bstart));
         GG_TRY(ensure(c, c->k2status, (size_t)ctiles * 8));
         GG_CUDA(cudaMemsetAsync(c->k2status.ptr, 0, (size_t)ctiles * 8, c->stream));
         gg::CountArgs ca{};
@@ -2049,10 +2061,7 @@ int grid_build_batched(grid_ctx *c, const grid_mesh *meshes, int32_t nmeshes, gr
         ca.mt = mt;
         ca.pair_base = pair_base_d;
         ca.bricks = may_brick;
-        if (may_brick) {
-            GG_TRY(ensure(c, c->bstart, (size_t)ntot * sizeof(unsigned)));
-            ca.bstart = (unsigned *)c->bstart.ptr;
-        }
+        ca.bstart = bstart;
         KernelScope ks(c, K_COUNT, 64.0 * ntot);
         GG_CUDA(gg::launch_count_scan(ca, c->stream));
     }
@@ -2094,8 +2103,7 @@ int grid_build_batched(grid_ctx *c, const grid_mesh *meshes, int32_t nmeshes, gr
             unsigned *tile_obj = (unsigned *)c->btile_obj.ptr;
             {
                 KernelScope ks(c, K_TILES, 4.0 * (ntiles + 1));
-                GG_CUDA(gg::launch_tile_search((const unsigned *)c->bstart.ptr, 1, ntot, gg::PAIR_TILE, ntiles,
-                                               tile_obj, c->stream));
+                GG_CUDA(gg::launch_tile_search(bstart, 1, ntot, gg::PAIR_TILE, ntiles, tile_obj, c->stream));
             }
             gg::BrickArgs ba{};
             ba.kb = bg.kb;
