@@ -150,6 +150,7 @@ __device__ __forceinline__ unsigned brick_start(const BrickArgs &a, unsigned b)
 // visits them, to write their zeros.
 __global__ void __launch_bounds__(256) brick_split_kernel(BrickArgs a)
 {
+    after_stream();
     __shared__ unsigned s_start[257];
     __shared__ unsigned s_tmp[8];
     __shared__ unsigned s_base, s_ebase, s_wbase;
@@ -358,6 +359,7 @@ __device__ __forceinline__ void finish_counts(const BrickArgs &a, const BrickIte
 template <bool CULLED>
 __global__ void __launch_bounds__(32 * COUNT_WARPS, 8) brick_count_kernel(BrickArgs a)
 {
+    after_stream();
     const unsigned lane = threadIdx.x & 31u;
     const unsigned nitems = min(ld_relaxed_u32(&a.ctl->tickets[3]), a.max_items);
     const unsigned nempty = min(ld_relaxed_u32(&a.ctl->tickets[6]), a.max_items);
@@ -416,6 +418,7 @@ constexpr int CULL_TRI = 25;   // words per triangle in shared memory (24 and a 
 
 __global__ void __launch_bounds__(32 * CULL_WARPS, 7) brick_cull_kernel(BrickArgs a)
 {
+    after_stream();
     __shared__ unsigned s_keep[CULL_WARPS][BRICK_CELLS];   // per cell: the word's kept entries; zero between words
     __shared__ float s_tri[CULL_WARPS][32 * CULL_TRI];
     __shared__ unsigned short s_list[CULL_WARPS][CULL_LIST];   // (entry's lane, cell) of pairs to test
@@ -720,6 +723,7 @@ __device__ __forceinline__ void store_offsets(const BrickArgs &a, long long p, c
 // into offsets.
 __global__ void __launch_bounds__(SCAN_BLOCK) cell_sums_kernel(BrickArgs a, unsigned ntiles)
 {
+    after_stream();
     __shared__ unsigned s_warp[SCAN_WARPS];
     __shared__ unsigned s_last;
     unsigned *sums = reinterpret_cast<unsigned *>(a.status);
@@ -768,6 +772,7 @@ __global__ void __launch_bounds__(SCAN_BLOCK) cell_sums_kernel(BrickArgs a, unsi
 template <int J, bool LOOKBACK>
 __global__ void __launch_bounds__(SCAN_BLOCK) cell_scan_kernel(BrickArgs a)
 {
+    after_stream();
     __shared__ unsigned s_tile;
     __shared__ unsigned s_warp[SCAN_WARPS];
     __shared__ unsigned s_excl;
@@ -916,6 +921,7 @@ __device__ __forceinline__ void stage_objects(unsigned *stage, const unsigned *s
 template <unsigned STAGE, int MIN_BLOCKS, bool CULLED, bool DENSE>
 __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel(BrickArgs a)
 {
+    after_stream();
     static_assert(STAGE >= 1024, "one word of 32 cells fits");
     constexpr unsigned W = FILL_WARPS;
     __shared__ __align__(16) unsigned s_mask[CULLED ? 4 : BRICK_CHUNK / 32 * MASK_PITCH];   // [word][feature]
@@ -1150,7 +1156,7 @@ unsigned long long cell_scan_tiles(long long ncells_out)
 
 cudaError_t launch_brick_split(const BrickArgs &a, cudaStream_t s)
 {
-    brick_split_kernel<<<(a.nbricks + 255u) / 256u, 256, 0, s>>>(a);
+    launch_after(brick_split_kernel, (a.nbricks + 255u) / 256u, 256, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -1159,9 +1165,9 @@ cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s)
     const unsigned blocks = (a.max_items + COUNT_WARPS - 1u) / COUNT_WARPS, cap = (unsigned)nsm * 64u;
     const unsigned grid = blocks < cap ? blocks : cap;
     if (a.masks)
-        brick_count_kernel<true><<<grid, 32 * COUNT_WARPS, 0, s>>>(a);
+        launch_after(brick_count_kernel<true>, grid, 32 * COUNT_WARPS, 0, s, a);
     else
-        brick_count_kernel<false><<<grid, 32 * COUNT_WARPS, 0, s>>>(a);
+        launch_after(brick_count_kernel<false>, grid, 32 * COUNT_WARPS, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -1169,10 +1175,10 @@ cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s)
 {
     const unsigned tiles = (unsigned)cell_scan_tiles(a.ncells_out);
     if (a.ncells_out > SCAN_ONE_PASS) {
-        cell_sums_kernel<<<tiles, SCAN_BLOCK, 0, s>>>(a, tiles);
-        cell_scan_kernel<SCAN_J, false><<<tiles, SCAN_BLOCK, 0, s>>>(a);
+        launch_after(cell_sums_kernel, tiles, SCAN_BLOCK, 0, s, a, tiles);
+        launch_after(cell_scan_kernel<SCAN_J, false>, tiles, SCAN_BLOCK, 0, s, a);
     } else {
-        cell_scan_kernel<1, true><<<tiles, SCAN_BLOCK, 0, s>>>(a);
+        launch_after(cell_scan_kernel<1, true>, tiles, SCAN_BLOCK, 0, s, a);
     }
     return cudaGetLastError();
 }
@@ -1188,11 +1194,11 @@ cudaError_t launch_brick_fill(const BrickArgs &a, int nsm, cudaStream_t s)
     // per SM, 667 with a block per item
     const unsigned cap = (unsigned)nsm * 256u, grid = a.max_items < cap ? a.max_items : cap;
     if (a.masks)
-        brick_fill_kernel<1024, 10, true, false><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+        launch_after(brick_fill_kernel<1024, 10, true, false>, grid, 32 * FILL_WARPS, 0, s, a);
     else if ((double)a.nrefs > DENSE_PAIRS_PER_CELL * (double)a.ncells_out)
-        brick_fill_kernel<3072, 6, false, true><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+        launch_after(brick_fill_kernel<3072, 6, false, true>, grid, 32 * FILL_WARPS, 0, s, a);
     else
-        brick_fill_kernel<1024, 10, false, true><<<grid, 32 * FILL_WARPS, 0, s>>>(a);
+        launch_after(brick_fill_kernel<1024, 10, false, true>, grid, 32 * FILL_WARPS, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -1206,7 +1212,7 @@ unsigned brick_max_words(unsigned nbricks, unsigned count)
 cudaError_t launch_brick_cull(const BrickArgs &a, int nsm, cudaStream_t s)
 {
     const unsigned blocks = (a.max_words + CULL_WARPS - 1u) / CULL_WARPS, cap = (unsigned)nsm * 64u;
-    brick_cull_kernel<<<blocks < cap ? blocks : cap, 32 * CULL_WARPS, 0, s>>>(a);
+    launch_after(brick_cull_kernel, blocks < cap ? blocks : cap, 32 * CULL_WARPS, 0, s, a);
     return cudaGetLastError();
 }
 

@@ -324,6 +324,7 @@ __global__ void __launch_bounds__(256, 8) bounds_kernel(const float *__restrict_
                                                      const int *__restrict__ tris, long long n,
                                                      Ctl *ctl, BoundsExtra x)
 {
+    after_stream();
 #pragma unroll
     for (int k = 0; k < 3; ++k)
         for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < x.zero[k].words; i += gridDim.x * blockDim.x)
@@ -416,6 +417,7 @@ __global__ void __launch_bounds__(256, 8) bounds_kernel(const float *__restrict_
 template <int BLOCK, int ITEMS, bool BRICKS>
 __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(CountArgs a)
 {
+    after_stream();
     constexpr int T = BLOCK * ITEMS;
     // one pad per thread's run: its ITEMS words in a row take 16 lanes each bank pair otherwise
     __shared__ unsigned long long s_pref[T + BLOCK];
@@ -613,12 +615,13 @@ __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(Cou
 
 __global__ void plan_kernel(Ctl *ctl, long long n, float lambda)
 {
+    after_stream();
     if (threadIdx.x == 0 && blockIdx.x == 0) device_plan(ctl, n, lambda);
 }
 
 cudaError_t launch_plan(Ctl *ctl, long long n, float lambda, cudaStream_t s)
 {
-    plan_kernel<<<1, 32, 0, s>>>(ctl, n, lambda);
+    launch_after(plan_kernel, 1, 32, 0, s, ctl, n, lambda);
     return cudaGetLastError();
 }
 
@@ -630,6 +633,7 @@ __global__ void __launch_bounds__(256) tile_search_kernel(const unsigned *__rest
                                                           unsigned tile, unsigned ntiles,
                                                           unsigned *__restrict__ tile_obj)
 {
+    after_stream();
     const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t > ntiles) return;
     if (t == ntiles) {
@@ -655,6 +659,7 @@ __global__ void __launch_bounds__(256) tile_search_kernel(const unsigned *__rest
 template <int BLOCK, int ITEMS>
 __global__ void __launch_bounds__(BLOCK) emit_kernel(EmitArgs a)
 {
+    after_stream();
     constexpr int T = BLOCK * ITEMS;
     extern __shared__ __align__(16) unsigned smem[];
     unsigned *s_mark = smem;                 // [padded T]
@@ -696,6 +701,7 @@ __global__ void __launch_bounds__(BLOCK) emit_kernel(EmitArgs a)
 template <int BLOCK, int ITEMS>
 __global__ void __launch_bounds__(BLOCK) cull_emit_kernel(CullArgs a)
 {
+    after_stream();
     constexpr int T = BLOCK * ITEMS;
     extern __shared__ __align__(16) unsigned smem[];
     unsigned *s_mark = smem;                     // [padded T]: object marks, then the tile's keys
@@ -911,6 +917,7 @@ template <int BLOCK, int ITEMS, int RBITS, int SRC>
 __global__ void __launch_bounds__(BLOCK, SRC != SRC_MEM ? gen_min_blocks<BLOCK>() : 2048 / BLOCK)
     upsweep_kernel(UpArgs a)
 {
+    after_stream();
     constexpr int T = BLOCK * ITEMS;
     constexpr int R = 1 << RBITS;
     extern __shared__ __align__(16) unsigned smem[];
@@ -1139,6 +1146,7 @@ __device__ __forceinline__ bool mbar_wait_phase0(unsigned long long *bar)
 template <int BLOCK, int ITEMS, int RBITS, int IN, bool STABLE>
 __global__ void __launch_bounds__(BLOCK, pass_min_blocks<BLOCK>()) downsweep_kernel(DownArgs a, unsigned gtiles)
 {
+    after_stream();
     constexpr int W = BLOCK / 32;
     constexpr int T = BLOCK * ITEMS;
     constexpr int R = 1 << RBITS;
@@ -1402,6 +1410,7 @@ __device__ __forceinline__ unsigned long long merge_split(const unsigned *keys, 
 // The split of every extraction block's first diagonal, all in parallel.
 __global__ void __launch_bounds__(256) extract_split_kernel(ExtractArgs a, unsigned long long nblocks)
 {
+    after_stream();
     const unsigned long long b = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (b > nblocks) return;
     const unsigned long long nA = a.count, nB = a.ncells + 1ull;
@@ -1414,6 +1423,7 @@ __global__ void __launch_bounds__(256) extract_split_kernel(ExtractArgs a, unsig
 template <int BLOCK, int ITEMS>
 __global__ void __launch_bounds__(BLOCK) extract_kernel(ExtractArgs a)
 {
+    after_stream();
     constexpr int D = BLOCK * ITEMS;
     static_assert((D & (D - 1)) == 0, "the lower-bound steps halve from D");
     __shared__ unsigned s_keys[D];
@@ -1540,6 +1550,7 @@ __device__ __forceinline__ unsigned bucket_start(const LocalArgs &a, unsigned b)
 // them once, shares them in shared memory, and opens the groups.
 __global__ void __launch_bounds__(256) bucket_split_kernel(LocalArgs a)
 {
+    after_stream();
     __shared__ unsigned s_st[256 + 2];   // starts of buckets b0 - 1 .. b0 + 256
     const unsigned b0 = blockIdx.x * 256u, b = b0 + threadIdx.x;
     if (b <= a.nbuckets) s_st[threadIdx.x + 1] = bucket_start(a, b);
@@ -1670,6 +1681,7 @@ __device__ __forceinline__ void l2_prefetch_u32(const unsigned *p, unsigned coun
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK, LOCAL_MIN_BLOCKS) local_sort_kernel(LocalArgs a)
 {
+    after_stream();
     constexpr int HN = 1 << LOCAL_LMAX;
     constexpr int PER = HN / BLOCK;   // cells per thread in the scan
     static_assert(HN % BLOCK == 0 && PER >= 1, "cells per thread");
@@ -1880,6 +1892,7 @@ constexpr int BOUNDS_ITEMS = 8;
 
 __global__ void __launch_bounds__(256) bounds_batched_kernel(MeshTab mt, long long ntot, unsigned *bstate, Ctl *ctl)
 {
+    after_stream();
     __shared__ int s_m0, s_m1;
     __shared__ unsigned s_lo[3], s_hi[3];
     const long long base = (long long)blockIdx.x * (256 * BOUNDS_ITEMS);
@@ -1990,6 +2003,7 @@ __global__ void __launch_bounds__(256) localize_kernel(const unsigned *__restric
                                                        const unsigned *__restrict__ pair_base, int nm,
                                                        long long total, unsigned *__restrict__ out)
 {
+    after_stream();
     const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= total) return;
     int lo = 0, hi = nm - 1;   // mesh m: largest with cells_off[m] <= q (every slice is non-empty)
@@ -2010,6 +2024,7 @@ __global__ void __launch_bounds__(256) rebase_recs_kernel(ObjRec *__restrict__ r
                                                           const long long *__restrict__ seg_obj0,
                                                           const unsigned *__restrict__ seg_p0, int nseg)
 {
+    after_stream();
     const long long o = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= n) return;
     int lo = 0, hi = nseg - 1;   // largest s with seg_obj0[s] <= o
@@ -2039,7 +2054,7 @@ cudaError_t launch_bounds(const float *verts, long long nverts, const int *tris,
     if (x) e = *x;
     if (blocks > 4 * nsm) e.plan = false;   // beyond, the blocks' atomics cost more than the launch
     if (planned) *planned = e.plan;
-    bounds_kernel<<<(unsigned)blocks, 256, 0, s>>>(verts, nverts, tris, n, ctl, e);
+    launch_after(bounds_kernel, (unsigned)blocks, 256, 0, s, verts, nverts, tris, n, ctl, e);
     return cudaGetLastError();
 }
 
@@ -2047,7 +2062,7 @@ cudaError_t launch_bounds_batched(const MeshTab &mt, long long ntot, unsigned *b
 {
     if (ntot <= 0) return cudaSuccess;
     const long long per_block = 256ll * BOUNDS_ITEMS;
-    bounds_batched_kernel<<<(unsigned)((ntot + per_block - 1) / per_block), 256, 0, s>>>(mt, ntot, bstate, ctl);
+    launch_after(bounds_batched_kernel, (unsigned)((ntot + per_block - 1) / per_block), 256, 0, s, mt, ntot, bstate, ctl);
     return cudaGetLastError();
 }
 
@@ -2055,7 +2070,7 @@ cudaError_t launch_localize(const unsigned *G, const long long *cells_off, const
                             long long total, unsigned *out, cudaStream_t s)
 {
     if (total <= 0) return cudaSuccess;
-    localize_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(G, cells_off, pair_base, nm, total, out);
+    launch_after(localize_kernel, (unsigned)((total + 255) / 256), 256, 0, s, G, cells_off, pair_base, nm, total, out);
     return cudaGetLastError();
 }
 
@@ -2063,7 +2078,7 @@ cudaError_t launch_rebase_recs(ObjRec *recs, long long n, const long long *seg_o
                                cudaStream_t s)
 {
     if (n <= 0 || nseg < 1) return cudaSuccess;
-    rebase_recs_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(recs, n, seg_obj0, seg_p0, nseg);
+    launch_after(rebase_recs_kernel, (unsigned)((n + 255) / 256), 256, 0, s, recs, n, seg_obj0, seg_p0, nseg);
     return cudaGetLastError();
 }
 
@@ -2072,9 +2087,9 @@ cudaError_t launch_count_scan(const CountArgs &a, cudaStream_t s)
     if (a.n <= 0) return cudaSuccess;
     const long long tiles = (a.n + COUNT_TILE - 1) / COUNT_TILE;
     if (a.bricks)
-        count_scan_kernel<COUNT_BLOCK, COUNT_TILE / COUNT_BLOCK, true><<<(unsigned)tiles, COUNT_BLOCK, 0, s>>>(a);
+        launch_after(count_scan_kernel<COUNT_BLOCK, COUNT_TILE / COUNT_BLOCK, true>, (unsigned)tiles, COUNT_BLOCK, 0, s, a);
     else
-        count_scan_kernel<COUNT_BLOCK, COUNT_TILE / COUNT_BLOCK, false><<<(unsigned)tiles, COUNT_BLOCK, 0, s>>>(a);
+        launch_after(count_scan_kernel<COUNT_BLOCK, COUNT_TILE / COUNT_BLOCK, false>, (unsigned)tiles, COUNT_BLOCK, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -2097,7 +2112,7 @@ cudaError_t launch_tile_search(const unsigned *starts, int stride, long long n, 
                                unsigned *tile_obj, cudaStream_t s)
 {
     const unsigned blocks = (ntiles + 1 + 255) / 256;
-    tile_search_kernel<<<blocks, 256, 0, s>>>(starts, stride, n, tile, ntiles, tile_obj);
+    launch_after(tile_search_kernel, blocks, 256, 0, s, starts, stride, n, tile, ntiles, tile_obj);
     return cudaGetLastError();
 }
 
@@ -2109,7 +2124,7 @@ cudaError_t launch_emit(const EmitArgs &a, cudaStream_t s)
     const size_t smem = 2 * sizeof(unsigned) * padded<PAIR_TILE>();
     static std::atomic<unsigned long long> configured{0};
     if (cudaError_t e = allow_dynamic_smem(k, smem, configured)) return e;
-    k<<<tiles, PAIR_BLOCK, smem, s>>>(a);
+    launch_after(k, tiles, PAIR_BLOCK, smem, s, a);
     return cudaGetLastError();
 }
 
@@ -2127,7 +2142,7 @@ cudaError_t launch_cull_emit(const CullArgs &a, cudaStream_t s)
     const size_t smem = 4 * sizeof(unsigned) * padded<PAIR_TILE>();
     static std::atomic<unsigned long long> configured{0};
     if (cudaError_t e = allow_dynamic_smem(k, smem, configured)) return e;
-    k<<<tiles, PAIR_BLOCK, smem, s>>>(a);
+    launch_after(k, tiles, PAIR_BLOCK, smem, s, a);
     return cudaGetLastError();
 }
 
@@ -2141,7 +2156,7 @@ static cudaError_t launch_up_t(const UpArgs &a, cudaStream_t s)
     if (cudaError_t e = allow_dynamic_smem(k, smem, configured)) return e;
     if (a.gtiles < 1 || a.gtiles > (unsigned)GROUP_TILES) return cudaErrorInvalidValue;
     const unsigned groups = (a.ntiles + a.gtiles - 1) / a.gtiles;
-    k<<<groups, BLOCK, smem, s>>>(a);
+    launch_after(k, groups, BLOCK, smem, s, a);
     return cudaGetLastError();
 }
 
@@ -2153,7 +2168,7 @@ static cudaError_t launch_down_t(const DownArgs &a, unsigned ntiles, unsigned gt
     constexpr size_t smem = down_smem_bytes<BLOCK, ITEMS, RBITS>();
     static std::atomic<unsigned long long> configured{0};
     if (cudaError_t e = allow_dynamic_smem(k, smem, configured)) return e;
-    k<<<ntiles, BLOCK, smem, s>>>(a, gtiles);
+    launch_after(k, ntiles, BLOCK, smem, s, a, gtiles);
     return cudaGetLastError();
 }
 
@@ -2224,7 +2239,7 @@ cudaError_t launch_downsweep(const DownArgs &a, int rbits, int in, unsigned ntil
 
 cudaError_t launch_bucket_split(const LocalArgs &a, cudaStream_t s)
 {
-    bucket_split_kernel<<<(a.nbuckets + 1 + 255) / 256, 256, 0, s>>>(a);
+    launch_after(bucket_split_kernel, (a.nbuckets + 1 + 255) / 256, 256, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -2242,7 +2257,7 @@ cudaError_t launch_local_sort(const LocalArgs &a, cudaStream_t s)
     if (cudaError_t e = cudaGetDevice(&dev)) return e;
     if (cudaError_t e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) return e;
     const unsigned grid = min(a.max_groups, (unsigned)(nsm * LOCAL_MIN_BLOCKS * 4));
-    k<<<grid, LOCAL_BLOCK, smem, s>>>(a);
+    launch_after(k, grid, LOCAL_BLOCK, smem, s, a);
     return cudaGetLastError();
 }
 
@@ -2254,14 +2269,14 @@ unsigned long long extract_blocks(unsigned long long count, unsigned long long n
 cudaError_t launch_extract_split(const ExtractArgs &a, cudaStream_t s)
 {
     const unsigned long long nb = extract_blocks(a.count, a.ncells);
-    extract_split_kernel<<<(unsigned)((nb + 1 + 255) / 256), 256, 0, s>>>(a, nb);
+    launch_after(extract_split_kernel, (unsigned)((nb + 1 + 255) / 256), 256, 0, s, a, nb);
     return cudaGetLastError();
 }
 
 cudaError_t launch_extract(const ExtractArgs &a, cudaStream_t s)
 {
     const unsigned long long nb = extract_blocks(a.count, a.ncells);
-    extract_kernel<EXTRACT_BLOCK, EXTRACT_TILE / EXTRACT_BLOCK><<<(unsigned)nb, EXTRACT_BLOCK, 0, s>>>(a);
+    launch_after(extract_kernel<EXTRACT_BLOCK, EXTRACT_TILE / EXTRACT_BLOCK>, (unsigned)nb, EXTRACT_BLOCK, 0, s, a);
     return cudaGetLastError();
 }
 
