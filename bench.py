@@ -161,13 +161,13 @@ def peaks():
 
 def kernels_digest() -> str:
     """First 16 hex digits of the sha256 of the kernels' code (csrc/kernels.cu,
-    kernels.h and device.cuh, in that order) with comments and whitespace
+    bricks.cu, cull.cuh, kernels.h and device.cuh, in that order) with comments and whitespace
     removed: a comment edit keeps the committed profiles valid, any code
     change does not."""
     import hashlib
     import re
     src = ""
-    for name in ("kernels.cu", "kernels.h", "device.cuh"):
+    for name in ("kernels.cu", "bricks.cu", "cull.cuh", "kernels.h", "device.cuh"):
         path = os.path.join(ROOT, "paper_2403_10647_gb300", "csrc", name)
         if os.path.exists(path):
             with open(path) as f:

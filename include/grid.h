@@ -118,7 +118,11 @@ typedef struct {
                              passes over the high key bits only, then one counting sort per bucket
                              of 2^L consecutive cells in shared memory, which also writes the
                              bucket's cell ranges.  The chain: radix passes over every key bit,
-                             then range extraction (the paper's).  0 (default): the hybrid at up to
+                             then range extraction (the paper's).  0 (default): with GRID_PAIRS_FUSED,
+                             bricks where they pay (from 2^21 pairs, and 4 pairs per brick entry, on):
+                             the radix passes sort one entry per 8 x 8 x 8 brick of cells and object
+                             instead of its pairs, and each brick's cells and refs are written from its
+                             entries; elsewhere the hybrid at up to
                              6 pairs per cell, with L chosen per build from the key width and the
                              pairs per cell, the chain otherwise.  -2: the hybrid always, L chosen
                              per build.  1..11: the hybrid always with that L (fewer radix passes,
@@ -157,9 +161,10 @@ const char *grid_version(void);
  * inputs read once, outputs written once).  Launches are counted always. */
 typedef struct {
     char name[32];        /* kernel family: bounds, count_scan, tile_search, emit, upsweep_gen,
-                             downsweep_gen, upsweep, downsweep, downsweep_first, extract_split,
-                             extract, bucket_split, local_sort, localize, make_pairs_per_object,
-                             cull_emit */
+                             downsweep_gen, upsweep, downsweep, downsweep_first, downsweep_keep,
+                             extract_split, extract, bucket_split (also the bricks' items), brick_count,
+                             cell_scan, local_sort (also the bricks' refs), localize,
+                             make_pairs_per_object, cull_emit (also the bricks' culling), plan, rebase */
     int64_t launches;
     double total_ms;      /* sum of event-timed durations (0 when profiling is off) */
     double bytes;         /* sum of algorithmic bytes */
@@ -189,7 +194,8 @@ int grid_ctx_autotune(grid_ctx *ctx, const float *verts, int64_t nverts, const i
  * gets L (the cell bits each per-bucket counting sort covers; -1 when every
  * key bit goes through radix passes, the paper's chain with range
  * extraction) and *passes the number of radix passes over the key bits
- * above L (may be NULL).  Host only. */
+ * above L (may be NULL).  Builds that take bricks (local_bits 0) do not use it.
+ * Host only. */
 int grid_ctx_sort_plan(grid_ctx *ctx, int32_t key_bits, int64_t count, int64_t ncells, int32_t *local_bits,
                        int32_t *passes);
 

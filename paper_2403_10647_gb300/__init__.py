@@ -135,7 +135,8 @@ class Context:
     def __init__(self, device: int = 0, radix_bits: int = 0, pair_gen: str = "fused", cull: bool = False,
                  tile_shape: str = "256x12", local_bits: int = 0):
         """local_bits: how builds finish the sort and the range steps (see
-        grid_opts.local_bits): 0 (default) = the hybrid (radix passes over the
+        grid_opts.local_bits): 0 (default) = bricks where they pay (radix passes over
+        (brick of cells, object) entries), elsewhere the hybrid (radix passes over the
         high key bits, then a per-bucket counting sort that also writes the
         cell ranges) at up to 6 pairs per cell, else radix passes over every
         key bit and range extraction; -2 = the hybrid always; 1..11 = the

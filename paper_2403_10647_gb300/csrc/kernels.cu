@@ -30,6 +30,9 @@
 //                        one problem.
 //   wait_selftest_kernel the radix sort's bounded look-back run against a
 //                        predecessor that never publishes (failure detection).
+// Builds by bricks (bricks.cu) use bounds, count_scan, upsweep and downsweep too:
+// the count scans their entries with the pairs, the first upsweep generates
+// entries instead of pairs.
 // The radix kernels are built for two block shapes (256 x 12 and 384 x 8
 // pairs per 3,072-pair tile) and for digits of 8 to 11 bits.
 #include <atomic>

@@ -257,7 +257,7 @@ int64_t estimate_bytes(int64_t pairs, int64_t ncells, int64_t n, int64_t nverts)
     return 4 * (ncells + 1) + 4 * pairs       // outputs
          + 28 * pairs + 4 * (ncells + 1)      // keys + values x2, sorted keys and values, object-order
                                               // pairs of the unfused modes, batch ranges
-         + 16 * n + 12 * nverts + (1 << 20);  // records, jittered vertices, small tables
+         + 20 * n + 12 * nverts + (1 << 20);  // records and first entries, jittered vertices, small tables
 }
 
 int grow(Worker *w, size_t bytes)
