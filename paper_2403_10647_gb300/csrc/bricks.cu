@@ -20,6 +20,12 @@
 // which of the 32 entries cover feature f; the entries covering cell (x, y, z)
 // are then X[x] & Y[y] & Z[z].  No atomics, no per-pair search, and ascending
 // bits are ascending objects.
+//
+// Measured, whole builds, sorted pairs then bricks: 10M-triangle building (2.4
+// pairs per cell, 2.0e8 pairs) 4.00 -> 1.72 ms; soup of 1M triangles (8.3e7 pairs)
+// 1.67 -> 0.33; soup of 7.3M (1.0e9 pairs) 22.7 -> 1.95; 64 soups (1.6e9 pairs)
+// 35.5 -> 3.6.  The pair path moved 12.8, 5.5, 70 and 91 GB for them, the
+// bricks 4.0, 0.6, 6.1 and 9.5.
 #include <atomic>
 #include <cstdint>
 
@@ -147,7 +153,8 @@ __device__ __forceinline__ unsigned brick_start(const BrickArgs &a, unsigned b)
 
 // One thread per brick: its first entry by binary search, its items appended to
 // the list.  Empty bricks go to the other end of the list: only the count
-// visits them, to write their zeros.
+// visits them, to write their zeros.  Bound by the searches' dependent loads
+// (21 us for 163,000 bricks).
 __global__ void __launch_bounds__(256) brick_split_kernel(BrickArgs a)
 {
     after_stream();
@@ -356,6 +363,12 @@ __device__ __forceinline__ void finish_counts(const BrickArgs &a, const BrickIte
 
 // A warp per item.  CULLED: the kept masks of its words instead of the boxes,
 // and their sum in ctl->nkept.
+//
+// Bound by the latency of an item's loads (its record, its entries, an object's
+// spilled box bits) with 8 blocks of 4 warps per SM, then by issue: 193 us at
+// 163,000 bricks (80M cells, 1.6e7 entries), 96 us at 59,000 bricks of crowded
+// cells.  More resident blocks spill (9, 10, 12 per SM: 189, 201, 206 us and 107,
+// 100, 120); 6 and 7 hide less (207, 205).
 template <bool CULLED>
 __global__ void __launch_bounds__(32 * COUNT_WARPS, 8) brick_count_kernel(BrickArgs a)
 {
@@ -410,6 +423,11 @@ __global__ void __launch_bounds__(32 * COUNT_WARPS, 8) brick_count_kernel(BrickA
 // below 4 u S W <= 24 u L^2 W for W >= max|w| over the brick; the plane's own
 // value here is off by no more.  T = S (1/2 + W 2^-16 + 2^-10) (1 + 2^-10) +
 // 2^-18 L^2 (L + W) exceeds R by the sum of these.
+//
+// Bound by issue (73% of cycles).  Tests and compaction pair by pair, ahead of a
+// sort of the pairs, then this kernel: 1150 -> 297 us on the soup of 1M triangles,
+// 764 -> 706 on a building of 2M.  A block per item instead of a warp per word:
+// 408 and 2038; rows of large boxes one lane each: 820 and 5018.
 constexpr int CULL_WARPS = 4;
 constexpr unsigned CULL_OWN = 16;
 constexpr unsigned CULL_LIST = 512;   // pairs listed for the test
@@ -589,13 +607,20 @@ __global__ void __launch_bounds__(32 * CULL_WARPS, 7) brick_cull_kernel(BrickArg
 // Up to SCAN_ONE_PASS cells: one pass, look-back between tiles.  Beyond, the
 // look-back's chain would set the time (32 tiles per round trip): a first
 // pass adds up each tile, its last block scans the sums, a second pass reads
-// the counts again, half of them from L2.
+// the counts again, half of them from L2 (80M cells: 165 us against 192 for
+// the look-back, in the forms of that time).
+//
+// Both passes wait on their loads: what helps is bytes in flight and few, long
+// blocks.  With SCAN_J_BIG loads per lane 80M cells take 123 us (J = 4: 149, 12:
+// 119, 16: 117) and 25M 49 us (J = 4: 56, 12: 52, 16: 53); 4M cells fill
+// the chip better with SCAN_J (16 us against 18), 8M take 22 us either way.
 constexpr int SCAN_BLOCK = 256;
 constexpr int SCAN_WARPS = SCAN_BLOCK / 32;
-constexpr long long SCAN_ONE_PASS = 1ll << 20;
-constexpr int SCAN_J = 4;   // loads per lane of the two passes
-constexpr long long SCAN_TILE = (long long)SCAN_BLOCK * 8 * SCAN_J;
-constexpr long long SCAN_SMALL_TILE = (long long)SCAN_BLOCK * 8;
+constexpr long long SCAN_ONE_PASS = 1ll << 20, SCAN_BIG = 1ll << 23;
+constexpr int SCAN_J = 4, SCAN_J_BIG = 8;   // loads per lane of the two passes
+
+template <int J>
+__host__ __device__ constexpr long long scan_tile() { return (long long)SCAN_BLOCK * 8 * J; }
 
 struct Counts8 {
     unsigned v[8];
@@ -685,6 +710,15 @@ __device__ __forceinline__ unsigned sum8(const Counts8 &c)
     return ((c.v[0] + c.v[1]) + (c.v[2] + c.v[3])) + ((c.v[4] + c.v[5]) + (c.v[6] + c.v[7]));
 }
 
+// Eight words at a multiple of 32 bytes (the cells arrays start on 256), whole sectors
+// at a time: as two 16-byte stores the scan took 172 against 151 us at 80M cells.
+__device__ __forceinline__ void store8(unsigned *p, const unsigned (&o)[8])
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                 "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7])
+                 : "memory");
+}
+
 // G of words p .. p + 7 from the sum x before them.
 __device__ __forceinline__ void store_offsets(const BrickArgs &a, long long p, const Counts8 &c, unsigned x, int m)
 {
@@ -709,9 +743,7 @@ __device__ __forceinline__ void store_offsets(const BrickArgs &a, long long p, c
         }
     }
     if (p + 8 <= a.ncells_out) {
-        uint4 *g = reinterpret_cast<uint4 *>(a.G + p);
-        g[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        g[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        store8(a.G + p, o);
     } else {
 #pragma unroll
         for (int k = 0; k < 8; ++k)
@@ -719,23 +751,68 @@ __device__ __forceinline__ void store_offsets(const BrickArgs &a, long long p, c
     }
 }
 
+// A warp's words [p, p + 256 J): `inner` when they lie inside one mesh's slice,
+// short of its last word, and no cell is on the list.  Their counts are then
+// the halves of the loaded words, and `base` is the mesh's first pair.
+struct WarpWords {
+    int m;   // mesh of word p
+    unsigned base;
+    bool inner;
+};
+
+template <int J>
+__device__ __forceinline__ WarpWords warp_words(const BrickArgs &a, long long p)
+{
+    WarpWords s{0, 0u, false};
+    long long end = a.ncells_out;
+    const unsigned nbig = ld_relaxed_u32(&a.ctl->tickets[1]);
+    if (a.mt.md && p < end) {
+        s.m = mesh_of_word(a, p);
+        end = __ldg(a.cells_off + s.m + 1);
+        s.base = __ldg(a.pair_base + s.m);
+    }
+    s.inner = nbig == 0u && p + 256 * J < end;
+    return s;
+}
+
+// The loads of load_raw where eight words are there.
+template <int J>
+__device__ __forceinline__ void load_words(const BrickArgs &a, long long p, uint4 (&raw)[J])
+{
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+        raw[j] = p + 256 * j + 8 <= a.ncells_out ? __ldcg(reinterpret_cast<const uint4 *>(a.counts + p + 256 * j))
+                                                 : make_uint4(0u, 0u, 0u, 0u);
+}
+
+__device__ __forceinline__ unsigned sum_halves(const uint4 &q)
+{
+    return __dp2a_lo(q.w, 0x0101u, __dp2a_lo(q.z, 0x0101u, __dp2a_lo(q.y, 0x0101u, __dp2a_lo(q.x, 0x0101u, 0u))));
+}
+
 // First pass: the sum of every tile; the last block to finish turns the sums
 // into offsets.
-__global__ void __launch_bounds__(SCAN_BLOCK) cell_sums_kernel(BrickArgs a, unsigned ntiles)
+template <int J>
+__global__ void __launch_bounds__(SCAN_BLOCK, J > SCAN_J ? 4 : 6) cell_sums_kernel(const __grid_constant__ BrickArgs a, unsigned ntiles)
 {
     after_stream();
     __shared__ unsigned s_warp[SCAN_WARPS];
     __shared__ unsigned s_last;
     unsigned *sums = reinterpret_cast<unsigned *>(a.status);
     const unsigned tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
-    const long long p0 = (long long)blockIdx.x * SCAN_TILE + (long long)w * (256 * SCAN_J) + 8 * lane;
-    uint4 raw[SCAN_J];
-#pragma unroll
-    for (int j = 0; j < SCAN_J; ++j) raw[j] = load_raw(a, p0 + 256 * j);
+    const long long pw = (long long)blockIdx.x * scan_tile<J>() + (long long)w * (256 * J), p0 = pw + 8 * lane;
+    uint4 raw[J];
+    load_words(a, p0, raw);
+    const WarpWords ww = warp_words<J>(a, pw);
     unsigned sum = 0u;
-    int m = a.mt.md ? mesh_of_word(a, p0) : 0;
+    if (ww.inner) {
 #pragma unroll
-    for (int j = 0; j < SCAN_J; ++j) sum += sum8(unpack(a, raw[j], p0 + 256 * j, &m));
+        for (int j = 0; j < J; ++j) sum += sum_halves(raw[j]);
+    } else {
+        int m = ww.m;
+#pragma unroll 1
+        for (int j = 0; j < J; ++j) sum += sum8(unpack(a, load_raw(a, p0 + 256 * j), p0 + 256 * j, &m));
+    }
     sum = __reduce_add_sync(FULL, sum);
     if (lane == 0u) s_warp[w] = sum;
     __syncthreads();
@@ -770,7 +847,7 @@ __global__ void __launch_bounds__(SCAN_BLOCK) cell_sums_kernel(BrickArgs a, unsi
 // The scan of one tile, from the first pass's offset or (LOOKBACK) from the
 // tiles before it.
 template <int J, bool LOOKBACK>
-__global__ void __launch_bounds__(SCAN_BLOCK) cell_scan_kernel(BrickArgs a)
+__global__ void __launch_bounds__(SCAN_BLOCK, J > SCAN_J ? 4 : 5) cell_scan_kernel(const __grid_constant__ BrickArgs a)
 {
     after_stream();
     __shared__ unsigned s_tile;
@@ -783,19 +860,24 @@ __global__ void __launch_bounds__(SCAN_BLOCK) cell_scan_kernel(BrickArgs a)
         __syncthreads();
         tile = s_tile;
     }
-    const long long p0 = (long long)tile * (SCAN_BLOCK * 8 * J) + (long long)w * (256 * J) + 8 * lane;
+    const long long pw = (long long)tile * scan_tile<J>() + (long long)w * (256 * J), p0 = pw + 8 * lane;
     uint4 raw[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) raw[j] = load_raw(a, p0 + 256 * j);
-    const int m0 = a.mt.md ? mesh_of_word(a, p0) : 0;
+    load_words(a, p0, raw);
+    const WarpWords ww = warp_words<J>(a, pw);
     unsigned off[J];   // words of the warp before this lane's load j
     unsigned run = 0u;
-    int m = m0;
+    if (ww.inner) {
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const unsigned sum = sum8(unpack(a, raw[j], p0 + 256 * j, &m)), inc = warp_incl_sum(sum);
-        off[j] = run + inc - sum;
-        run += __shfl_sync(FULL, inc, 31);
+        for (int j = 0; j < J; ++j) {
+            const unsigned sum = sum_halves(raw[j]), inc = warp_incl_sum(sum);
+            off[j] = run + inc - sum;
+            run += __shfl_sync(FULL, inc, 31);
+        }
+    } else {
+        int m = ww.m;
+#pragma unroll 1
+        for (int j = 0; j < J; ++j)
+            run += __reduce_add_sync(FULL, sum8(unpack(a, load_raw(a, p0 + 256 * j), p0 + 256 * j, &m)));
     }
     if (lane == 31u) s_warp[w] = run;
     __syncthreads();
@@ -812,12 +894,30 @@ __global__ void __launch_bounds__(SCAN_BLOCK) cell_scan_kernel(BrickArgs a)
         }
     }
     __syncthreads();
-    const unsigned base = s_excl + s_warp[w];
-    m = m0;
+    unsigned base = s_excl + s_warp[w];
+    if (ww.inner) {
+        base -= ww.base;
 #pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const unsigned c[4] = {raw[j].x, raw[j].y, raw[j].z, raw[j].w};
+            unsigned o[8];
+            o[0] = base + off[j];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                o[2 * k + 1] = o[2 * k] + (c[k] & 0xFFFFu);
+                if (k < 3) o[2 * k + 2] = o[2 * k + 1] + (c[k] >> 16);
+            }
+            store8(a.G + p0 + 256 * j, o);
+        }
+        return;
+    }
+    int m = ww.m;
+#pragma unroll 1
     for (int j = 0; j < J; ++j) {
-        const Counts8 c = unpack(a, raw[j], p0 + 256 * j, &m);
-        store_offsets(a, p0 + 256 * j, c, base + off[j], m);
+        const Counts8 c = unpack(a, load_raw(a, p0 + 256 * j), p0 + 256 * j, &m);
+        const unsigned sum = sum8(c), inc = warp_incl_sum(sum);
+        store_offsets(a, p0 + 256 * j, c, base + inc - sum, m);
+        base += __shfl_sync(FULL, inc, 31);
     }
 }
 
@@ -918,6 +1018,14 @@ __device__ __forceinline__ void stage_objects(unsigned *stage, const unsigned *s
 // run then, copied by whole warps without a tag, a lookup of its place and
 // one of its object per ref.  Shared memory bounds the fill there (91% of its
 // rate with tags): 1.47 -> 1.26 ms on the soup of 7.3M triangles, 1.0e9 refs.
+//
+// Bound by issue (78% of cycles) and shared memory (47 to 59% of its wavefronts);
+// device memory is at a quarter of its rate.  Masks alone, no pairs written: 0.25
+// of 0.64 ms at the 10M building.  One cell per lane 1.09, four 0.73 (one bit
+// search serves four lists), two refs per lane in flight and one range check per
+// cell 0.67, objects staged 0.66, the wider grid 0.64.  Measured and dropped: 16
+// warps per block, lanes walking words independently (0.92 against 0.73), a lane
+// per entry with popcount ranks (1.41), the next item's record loaded early.
 template <unsigned STAGE, int MIN_BLOCKS, bool CULLED, bool DENSE>
 __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel(BrickArgs a)
 {
@@ -1150,7 +1258,9 @@ unsigned brick_max_items(unsigned nbricks, unsigned count)
 
 unsigned long long cell_scan_tiles(long long ncells_out)
 {
-    const long long t = ncells_out > SCAN_ONE_PASS ? SCAN_TILE : SCAN_SMALL_TILE;
+    const long long t = ncells_out > SCAN_BIG        ? scan_tile<SCAN_J_BIG>()
+                        : ncells_out > SCAN_ONE_PASS ? scan_tile<SCAN_J>()
+                                                     : scan_tile<1>();
     return (unsigned long long)((ncells_out + t - 1) / t);
 }
 
@@ -1174,8 +1284,11 @@ cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s)
 cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s)
 {
     const unsigned tiles = (unsigned)cell_scan_tiles(a.ncells_out);
-    if (a.ncells_out > SCAN_ONE_PASS) {
-        launch_after(cell_sums_kernel, tiles, SCAN_BLOCK, 0, s, a, tiles);
+    if (a.ncells_out > SCAN_BIG) {
+        launch_after(cell_sums_kernel<SCAN_J_BIG>, tiles, SCAN_BLOCK, 0, s, a, tiles);
+        launch_after(cell_scan_kernel<SCAN_J_BIG, false>, tiles, SCAN_BLOCK, 0, s, a);
+    } else if (a.ncells_out > SCAN_ONE_PASS) {
+        launch_after(cell_sums_kernel<SCAN_J>, tiles, SCAN_BLOCK, 0, s, a, tiles);
         launch_after(cell_scan_kernel<SCAN_J, false>, tiles, SCAN_BLOCK, 0, s, a);
     } else {
         launch_after(cell_scan_kernel<1, true>, tiles, SCAN_BLOCK, 0, s, a);

@@ -98,3 +98,35 @@ def test_brick_batch_matches_oracle():
             assert_grid_equal(g, oracle.build_grid(s.verts, s.tris, s.lam, method="counting"), f"mesh {k}")
     finally:
         c.close()
+
+
+# cells on both sides of the scan's changes of tile; `crowd`: one cell beyond 16 bits
+@pytest.mark.parametrize("lam,crowd", [(50.0, 0), (54.0, 70_000), (414.0, 0), (430.0, 0), (95.0, 70_000)])
+def test_cell_scan_sizes_match_oracle(lam, crowd):
+    import paper_2403_10647_gb300 as pg
+    s = _soup(20_000, (10, 9.3, 11.1), 0.5, 41, lam, giants=2, crowd=crowd)
+    o = oracle.build_grid(s.verts, s.tris, s.lam, method="counting")
+    c = pg.Context(0)
+    try:
+        c.profile(True)
+        assert_grid_equal(c.build(dev(s.verts, torch.float32), dev(s.tris, torch.int32), s.lam), o, str(lam))
+        assert "cell_scan" in c.kernel_stats()
+    finally:
+        c.close()
+
+
+@pytest.mark.parametrize("lam", [30.0, 200.0])
+def test_cell_scan_of_a_batch_matches_oracle(lam):
+    """Slices shorter than a warp's words, between long ones that a warp lies in."""
+    import paper_2403_10647_gb300 as pg
+    batch = [_soup(k, (1, 2, 3), 0.5, 50 + k, 8.0) for k in (3, 1, 40)] + [_soup(20_000, (10, 9.3, 11.1), 0.7, 42, lam)]
+    batch += [_soup(k, (2, 1, 3), 0.5, 60 + k, 5.0) for k in (2, 300)] + [_soup(22_000, (9, 9.3, 8), 0.7, 43, lam)]
+    c = pg.Context(0)
+    try:
+        c.profile(True)
+        grids = c.build_batched([(dev(s.verts, torch.float32), dev(s.tris, torch.int32), s.lam) for s in batch])
+        assert "cell_scan" in c.kernel_stats()
+        for k, (s, g) in enumerate(zip(batch, grids)):
+            assert_grid_equal(g, oracle.build_grid(s.verts, s.tris, s.lam, method="counting"), f"mesh {k}")
+    finally:
+        c.close()
