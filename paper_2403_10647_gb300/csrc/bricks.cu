@@ -23,7 +23,7 @@
 //
 // Measured, whole builds, sorted pairs then bricks: 10M-triangle building (2.4
 // pairs per cell, 2.0e8 pairs) 4.00 -> 1.72 ms; soup of 1M triangles (8.3e7 pairs)
-// 1.67 -> 0.33; soup of 7.3M (1.0e9 pairs) 22.7 -> 1.95; 64 soups (1.6e9 pairs)
+// 1.68 -> 0.33; soup of 7.3M (1.0e9 pairs) 22.7 -> 1.95; 64 soups (1.6e9 pairs)
 // 35.5 -> 3.6.  The pair path moved 12.8, 5.5, 70 and 91 GB for them, the
 // bricks 4.0, 0.6, 6.1 and 9.5.
 #include <atomic>

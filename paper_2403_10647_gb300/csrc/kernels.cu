@@ -197,7 +197,10 @@ __device__ __forceinline__ void gen_blocked(const ObjRec *__restrict__ recs, uns
 
 // The same for a brick build: the thread's ITEMS consecutive entries (brick,
 // object) of the tile, x fastest over the bricks that the object's box meets,
-// each packed with the part of the box inside the brick (BrickGen).
+// each packed with the part of the box inside the brick (BrickGen).  Bound by
+// the record loads (an entry's object, then its box) at half the issue rate: the
+// generating upsweep takes 0.14 ms at 10M architectural triangles (1.6e7
+// entries), 0.63 for their 2.0e8 pairs.
 template <int ITEMS>
 __device__ __forceinline__ void gen_bricks(const ObjRec *__restrict__ recs, const unsigned *__restrict__ bstart,
                                            unsigned of, const unsigned (&om)[ITEMS], unsigned j0, unsigned cnt,
@@ -322,7 +325,8 @@ __device__ void device_plan(Ctl *ctl, long long n, float lambda)
 // ---------------------------------------------------------------------------
 
 // Compiled for 8 resident blocks per SM (32 registers): at the 36 that the
-// prefetch takes otherwise, a 5M-triangle mesh takes 48 us instead of 37.
+// prefetch takes otherwise, a 5M-triangle mesh takes 48 us instead of 37 (58
+// without the prefetch).  Bound by the vertex gathers (5.0 TB/s at 10M triangles).
 __global__ void __launch_bounds__(256, 8) bounds_kernel(const float *__restrict__ verts, long long nverts,
                                                      const int *__restrict__ tris, long long n,
                                                      Ctl *ctl, BoundsExtra x)
@@ -417,6 +421,11 @@ __global__ void __launch_bounds__(256, 8) bounds_kernel(const float *__restrict_
 // BRICKS: the bricks that an object's box meets are counted and scanned with
 // the pairs, in the bits from BRICK_SUM_BITS on, and the pairs added up once
 // more on their own, so that the host knows whether they overflowed theirs.
+//
+// Bound by the chain index load, vertex load, tile scan, look-back.  The next
+// triangle's indices loaded one ahead and a padded staging tile (bank conflicts were
+// 81% of its wavefronts): 212 -> 197 us at 10M triangles with the second sum,
+// 150 -> 139 at 7.3M; the vertices as one or two 16-byte loads each: 205.
 template <int BLOCK, int ITEMS, bool BRICKS>
 __global__ void __launch_bounds__(BLOCK, COUNT_MIN_BLOCKS) count_scan_kernel(CountArgs a)
 {
@@ -1889,8 +1898,8 @@ __global__ void __launch_bounds__(BLOCK, LOCAL_MIN_BLOCKS) local_sort_kernel(Loc
 // up once and the block updates it once; in other blocks a thread looks up
 // each triangle's mesh and updates it when it changes.  bstate[m * 6 + a] holds
 // ~ordered(min) for a < 3 and ordered(max) for a >= 3 (both atomicMax).
-// Bound by the index and vertex loads; with eight consecutive triangles per
-// thread and a look-up for each, 20.5M triangles took 0.51 ms.
+// Bound by the index and vertex loads: 20.5M triangles in 0.15 ms (6.6 TB/s); with
+// eight consecutive triangles per thread and a look-up for each they took 0.51.
 constexpr int BOUNDS_ITEMS = 8;
 
 __global__ void __launch_bounds__(256) bounds_batched_kernel(MeshTab mt, long long ntot, unsigned *bstate, Ctl *ctl)
