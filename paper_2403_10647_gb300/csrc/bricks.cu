@@ -151,27 +151,34 @@ __device__ __forceinline__ unsigned brick_start(const BrickArgs &a, unsigned b)
 // split: bricks -> work items
 // ---------------------------------------------------------------------------
 
-// One thread per brick: its first entry by binary search, its items appended to
-// the list.  Empty bricks go to the other end of the list: only the count
-// visits them, to write their zeros.  Bound by the searches' dependent loads
-// (21 us for 163,000 bricks).
-__global__ void __launch_bounds__(256) brick_split_kernel(BrickArgs a)
+// One thread per brick: its first entry by binary search.  The block then writes
+// its bricks' items (and, for culled builds, their words) one after another, a
+// thread per item, so that a brick of thousands of chunks takes no longer than
+// as many bricks: with each thread writing its own brick's, a brick of 4M entries
+// took 145 us (774 culled), now under 20 (76).  Empty bricks go to the other end of the
+// list: only the count visits them, to write their zeros.  Bound by the
+// searches' dependent loads (21 us for 163,000 bricks).
+constexpr unsigned SPLIT_BLOCK = 256;
+
+__global__ void __launch_bounds__(SPLIT_BLOCK) brick_split_kernel(BrickArgs a)
 {
     after_stream();
-    __shared__ unsigned s_start[257];
-    __shared__ unsigned s_tmp[8];
+    __shared__ unsigned s_start[SPLIT_BLOCK + 1];
+    __shared__ unsigned s_tmp[SPLIT_BLOCK / 32];
     __shared__ unsigned s_base, s_ebase, s_wbase;
-    const unsigned tid = threadIdx.x, b0 = blockIdx.x * 256u, b = b0 + tid;
+    __shared__ BrickItem s_item[SPLIT_BLOCK];       // the brick, its entries as one item; slot: the first chunk's
+    __shared__ unsigned s_iex[SPLIT_BLOCK], s_wex[SPLIT_BLOCK];   // items and words of the bricks before
+    const unsigned tid = threadIdx.x, b0 = blockIdx.x * SPLIT_BLOCK, b = b0 + tid;
     if (b <= a.nbricks) s_start[tid] = brick_start(a, b);
-    if (tid == 255u && b + 1u <= a.nbricks) s_start[256] = brick_start(a, b + 1u);
+    if (tid == SPLIT_BLOCK - 1u && b + 1u <= a.nbricks) s_start[SPLIT_BLOCK] = brick_start(a, b + 1u);
     __syncthreads();
     const bool ok = b < a.nbricks;
     BrickItem it{};
-    unsigned m = 0u, k = 0u;
+    unsigned k = 0u;
     if (ok) {
         it.first = s_start[tid];
-        m = s_start[tid + 1] - it.first;
-        k = (m + BRICK_CHUNK - 1u) / BRICK_CHUNK;
+        it.count = s_start[tid + 1] - it.first;
+        k = (it.count + BRICK_CHUNK - 1u) / BRICK_CHUNK;
         unsigned shape = a.shape, nbx = a.nbx, nby = a.nby, lb = b;
         int r[3] = {a.res[0], a.res[1], a.res[2]};
         unsigned long long c0 = 0ull;
@@ -196,60 +203,67 @@ __global__ void __launch_bounds__(256) brick_split_kernel(BrickArgs a)
         const unsigned ex = min(1u << lx, (unsigned)r[0] - x0) - 1u, ey = min(1u << ly, (unsigned)r[1] - y0) - 1u,
                        ez = min(1u << lz, (unsigned)r[2] - z0) - 1u;
         it.dims = ex | (ey << 5) | (ez << 10) | (lx << 15) | (ly << 18) | (lz << 21);
+        it.slot = k > 1u ? atomicAdd(&a.ctl->tickets[4], k) : NO_SLOT;
     }
-    unsigned total, etotal;
-    const unsigned ex = block_excl_sum<256>(k, s_tmp, &total);
-    const unsigned eex = block_excl_sum<256>(ok && m == 0u ? 1u : 0u, s_tmp, &etotal);
-    const unsigned words = a.masks && ok ? (m + 31u) / 32u : 0u;
-    unsigned wex = 0u, wtotal = 0u;
-    if (a.masks) wex = block_excl_sum<256>(words, s_tmp, &wtotal);
+    const bool empty = ok && k == 0u;
+    unsigned total, etotal, wtotal = 0u;
+    const unsigned iex = block_excl_sum<SPLIT_BLOCK>(k, s_tmp, &total);
+    const unsigned eex = block_excl_sum<SPLIT_BLOCK>(empty ? 1u : 0u, s_tmp, &etotal);
+    if (a.masks) s_wex[tid] = block_excl_sum<SPLIT_BLOCK>((it.count + 31u) / 32u, s_tmp, &wtotal);
+    s_item[tid] = it;
+    s_iex[tid] = iex;
     if (tid == 0u) {
         s_wbase = wtotal ? atomicAdd(&a.ctl->tickets[2], wtotal) : 0u;
         s_base = total ? atomicAdd(&a.ctl->tickets[3], total) : 0u;
         s_ebase = etotal ? atomicAdd(&a.ctl->tickets[6], etotal) : 0u;
     }
     __syncthreads();
-    if (ok && m == 0u) {
+    bool bad = false;   // never: the host sizes the lists for every split of `count` entries
+    if (empty) {
         const unsigned p = s_ebase + eex;
-        it.count = 0u;
-        it.slot = NO_SLOT;
         if (p < a.max_items)
             a.items[a.max_items - 1u - p] = it;
         else
-            atomicOr(&a.ctl->err, ERR_RANGE);
+            bad = true;
     }
-    if (k) {
-        unsigned slot = NO_SLOT;
-        if (k > 1u) {
-            slot = atomicAdd(&a.ctl->tickets[4], k);
-            if (slot + k <= a.max_slots)
-                a.arrive[slot] = 0u;
+    // the last brick of the block with before[q] <= i: the one that holds item (or word) i
+    auto brick_of = [](const unsigned *before, unsigned i) {
+        unsigned lo = 0u;
+#pragma unroll
+        for (unsigned step = SPLIT_BLOCK / 2u; step; step >>= 1)
+            if (before[lo + step] <= i) lo += step;
+        return lo;
+    };
+    for (unsigned i = tid; i < total; i += SPLIT_BLOCK) {
+        const unsigned q = brick_of(s_iex, i), j = i - s_iex[q], p = s_base + i;
+        BrickItem o = s_item[q];
+        const unsigned m = o.count, chunks = (m + BRICK_CHUNK - 1u) / BRICK_CHUNK, slot0 = o.slot;
+        o.first += j * BRICK_CHUNK;
+        o.count = min((unsigned)BRICK_CHUNK, m - j * BRICK_CHUNK);
+        if (chunks > 1u) {
+            o.slot = slot0 + j;
+            if (o.slot >= a.max_slots) {
+                bad = true;
+                continue;
+            }
+            a.slot_meta[o.slot] = make_uint2(slot0, chunks);
+            a.arrive[o.slot] = 0u;
         }
-        const unsigned p = s_base + ex;
-        // never beyond: the host sizes both lists for every split of `count` entries
-        if (p + k > a.max_items || (k > 1u && slot + k > a.max_slots)) {
-            atomicOr(&a.ctl->err, ERR_RANGE);
-        } else {
-            const unsigned first = it.first;
-            for (unsigned j = 0; j < k; ++j) {
-                it.first = first + j * BRICK_CHUNK;
-                it.count = min((unsigned)BRICK_CHUNK, m - j * BRICK_CHUNK);
-                it.slot = k > 1u ? slot + j : NO_SLOT;
-                if (k > 1u) a.slot_meta[slot + j] = make_uint2(slot, k);
-                a.items[p + j] = it;
-            }
-            if (a.masks) {
-                const unsigned w0 = s_wbase + wex;
-                if (w0 + words > a.max_words) {   // never: max_words bounds the words of all items
-                    atomicOr(&a.ctl->err, ERR_RANGE);
-                    for (unsigned j = 0; j < k; ++j) a.mask0[p + j] = 0u;
-                } else {
-                    for (unsigned j = 0; j < k; ++j) a.mask0[p + j] = w0 + j * (BRICK_CHUNK / 32);
-                    for (unsigned q = 0; q < words; ++q) a.word_item[w0 + q] = p + q / (BRICK_CHUNK / 32);
-                }
-            }
+        if (p >= a.max_items) {
+            bad = true;
+            continue;
+        }
+        a.items[p] = o;
+        if (a.masks) {
+            const unsigned w0 = s_wbase + s_wex[q] + j * (BRICK_CHUNK / 32), words = (o.count + 31u) / 32u;
+            const bool fits = w0 + words <= a.max_words;
+            a.mask0[p] = fits ? w0 : 0u;
+            if (fits)
+                for (unsigned w = 0; w < words; ++w) a.word_item[w0 + w] = p;
+            bad |= !fits;
         }
     }
+    if (bad) atomicOr(&a.ctl->err, ERR_RANGE);
 }
 
 // ---------------------------------------------------------------------------
