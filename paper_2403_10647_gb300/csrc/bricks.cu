@@ -312,10 +312,62 @@ __device__ __forceinline__ void count_words(const BrickArgs &a, const BrickItem 
     }
 }
 
+// Rows of a brick in k > 1 chunks: its chunks' counts at slots [s, s + k) and, when
+// k > MERGE_CHUNKS, the sums of merge_group(k) chunks each at group_row.
+constexpr unsigned MERGE_CHUNKS = 32;
+
+// The smallest power of two whose square is at least k, 16 at the least.
+__host__ __device__ __forceinline__ unsigned merge_group(unsigned k)
+{
+    unsigned g = 16u;
+    while (g < 65536u && g * g < k) g <<= 1;
+    return g;
+}
+
+// First of a brick's group rows, behind the max_slots chunk rows: more than
+// MERGE_CHUNKS chunks make at most k / 8 groups, so the rows of two bricks
+// (their slots follow one another) stay apart.
+__device__ __forceinline__ unsigned group_row(const BrickArgs &a, unsigned slot0) { return a.max_slots + (slot0 + 7u) / 8u; }
+
+// Turns n rows of counts into offsets (each the sum of the rows before) and
+// adds them up in cnt (one warp; lane l of group g has cell 32 g + l).
+__device__ __forceinline__ void scan_rows(unsigned *rows, unsigned n, unsigned (&cnt)[GROUPS])
+{
+    const unsigned lane = threadIdx.x & 31u;
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) cnt[g] = 0u;
+    for (unsigned j = 0; j < n; ++j) {
+        unsigned *row = rows + (size_t)j * BRICK_CELLS + lane, v[GROUPS];
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) v[g] = __ldcg(row + 32 * g);
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) {
+            row[32 * g] = cnt[g];
+            cnt[g] += v[g];
+        }
+    }
+}
+
+// One more of n arrivals at *count: is it the last?  What the warps that
+// arrived before wrote is visible to the last.
+__device__ __forceinline__ bool last_to_arrive(unsigned *count, unsigned n)
+{
+    __threadfence();
+    __syncwarp();
+    unsigned last = 0u;
+    if ((threadIdx.x & 31u) == 0u) last = atomicAdd(count, 1u) + 1u == n;
+    last = __shfl_sync(FULL, last, 0);
+    if (last) __threadfence();
+    return last;
+}
+
 // Writes an item's counts (lane l of group g has cell 32 g + l; one warp).  A
 // brick in one item writes its cells' counts; a chunk writes its own to its
 // slot, and the last chunk of the brick to arrive turns the slots into offsets
-// inside each cell and writes the sums.
+// inside each cell and writes the sums.  A slot costs that warp a round trip to
+// L2 (0.24 us), so a brick of more than MERGE_CHUNKS chunks is added up in two
+// levels: the last chunk of each group to arrive does the group's slots, the
+// last group the groups' sums.
 __device__ __forceinline__ void finish_counts(const BrickArgs &a, const BrickItem &it, const Dims &d,
                                               unsigned (&cnt)[GROUPS])
 {
@@ -324,26 +376,21 @@ __device__ __forceinline__ void finish_counts(const BrickArgs &a, const BrickIte
         unsigned *sl = a.slots + (size_t)it.slot * BRICK_CELLS;
 #pragma unroll
         for (int g = 0; g < GROUPS; ++g) sl[32 * g + lane] = cnt[g];
-        const uint2 meta = a.slot_meta[it.slot];
-        __threadfence();
-        __syncwarp();
-        unsigned last = 0u;
-        if (lane == 0u) last = atomicAdd(a.arrive + meta.x, 1u) + 1u == meta.y;
-        if (!__shfl_sync(FULL, last, 0)) return;
-        __threadfence();
-        // every chunk of the brick is counted: offsets of the chunks inside each cell
+        const uint2 meta = a.slot_meta[it.slot];   // the brick's first slot, its chunks
+        bool top = meta.y <= MERGE_CHUNKS;
+        const unsigned per = top ? meta.y : merge_group(meta.y), q = (it.slot - meta.x) / per;
+        unsigned row0 = meta.x + q * per, n = min(per, meta.y - q * per), *arrive = a.arrive + row0;
+        for (;;) {
+            if (!last_to_arrive(arrive, n)) return;
+            scan_rows(a.slots + (size_t)row0 * BRICK_CELLS, n, cnt);
+            if (top) break;
+            top = true;
+            row0 = group_row(a, meta.x);
+            n = (meta.y + per - 1u) / per;
+            arrive = a.arrive + meta.x + 1u;   // no group starts at a brick's second slot
+            unsigned *sum = a.slots + (size_t)(row0 + q) * BRICK_CELLS + lane;
 #pragma unroll
-        for (int g = 0; g < GROUPS; ++g) cnt[g] = 0u;
-        for (unsigned j = 0; j < meta.y; ++j) {
-            unsigned *sj = a.slots + (size_t)(meta.x + j) * BRICK_CELLS;
-            unsigned v[GROUPS];
-#pragma unroll
-            for (int g = 0; g < GROUPS; ++g) v[g] = __ldcg(sj + 32 * g + lane);
-#pragma unroll
-            for (int g = 0; g < GROUPS; ++g) {
-                sj[32 * g + lane] = cnt[g];
-                cnt[g] += v[g];
-            }
+            for (int g = 0; g < GROUPS; ++g) sum[32 * g] = cnt[g];
         }
     }
     unsigned most = 0u;
@@ -1068,6 +1115,15 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
         unsigned dst[4], num[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) dst[k] = num[k] = 0u;
+        // a chunk's rows: the brick's chunks before it come first in each cell
+        const unsigned *before = nullptr, *before_group = nullptr;
+        if (it.slot != NO_SLOT) {
+            const uint2 meta = a.slot_meta[it.slot];
+            before = a.slots + (size_t)it.slot * BRICK_CELLS + c0;
+            if (meta.y > MERGE_CHUNKS)
+                before_group = a.slots + c0 +
+                               (size_t)(group_row(a, meta.x) + (it.slot - meta.x) / merge_group(meta.y)) * BRICK_CELLS;
+        }
         if (y < d.ny && z < d.nz) {
             const unsigned *gp = a.G + it.cell0 + x + it.rx * y + it.rxy * z;
             unsigned g[5];
@@ -1079,8 +1135,9 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
                     dst[k] = it.base + g[k];
                     num[k] = g[k + 1] - g[k];
                     bad |= num[k] > a.nrefs || dst[k] > a.nrefs - num[k];
-                    // the cell's other chunks come first; this one's share is counted below
-                    if (it.slot != NO_SLOT) dst[k] += __ldg(a.slots + (size_t)it.slot * BRICK_CELLS + c0 + k);
+                    // this chunk's share of the cell is counted below
+                    if (before) dst[k] += __ldg(before + k);
+                    if (before_group) dst[k] += __ldg(before_group + k);
                 }
             }
         }
@@ -1263,6 +1320,9 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
 // A brick in k > 1 chunks holds more than (k - 1) BRICK_CHUNK entries, at least
 // k BRICK_CHUNK / 2.
 unsigned brick_max_slots(unsigned count) { return 2u * (count / BRICK_CHUNK) + 2u; }
+
+// Group rows behind the slots (group_row).
+unsigned brick_max_groups(unsigned count) { return brick_max_slots(count) / 8u + 2u; }
 
 unsigned brick_max_items(unsigned nbricks, unsigned count)
 {

@@ -367,8 +367,11 @@ struct BrickArgs {
     unsigned max_items;
     unsigned max_slots;
     unsigned *slots;                // [max_slots][BRICK_CELLS]: a chunk's counts, then its offsets in the cells
+                                    // (its group's, of a brick in many chunks); then [brick_max_groups]
+                                    // such rows of groups of chunks
     uint2 *slot_meta;               // [max_slots]: the brick's first slot and its number of slots
-    unsigned *arrive;               // [max_slots]: chunks counted, at the brick's first slot
+    unsigned *arrive;               // [max_slots]: chunks counted, at the brick's (or group's) first slot;
+                                    // groups counted, at the brick's second
     unsigned short *counts;         // [ncells_out] objects per cell; BRICK_BIG and more: in `big`
     uint2 *big;                     // [max_big]: cell, objects
     unsigned max_big;
@@ -392,6 +395,7 @@ struct BrickArgs {
 constexpr unsigned BRICK_BIG = 65535u;
 
 unsigned brick_max_slots(unsigned count);
+unsigned brick_max_groups(unsigned count);
 unsigned brick_max_items(unsigned nbricks, unsigned count);
 unsigned long long cell_scan_tiles(long long ncells_out);
 cudaError_t launch_brick_split(const BrickArgs &a, cudaStream_t s);

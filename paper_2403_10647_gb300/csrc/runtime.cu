@@ -784,7 +784,7 @@ int sort_bricks(grid_ctx *c, gg::BrickArgs &a, const gg::BrickGen &bg, unsigned 
     a.max_slots = gg::brick_max_slots(entries);
     a.max_big = a.nrefs / gg::BRICK_BIG + 1u;
     const size_t sizes[6] = {(size_t)a.max_items * sizeof(gg::BrickItem),
-                             (size_t)a.max_slots * gg::BRICK_CELLS * sizeof(unsigned),
+                             ((size_t)a.max_slots + gg::brick_max_groups(entries)) * gg::BRICK_CELLS * sizeof(unsigned),
                              (size_t)a.max_slots * sizeof(uint2),
                              (size_t)a.max_slots * sizeof(unsigned),
                              (size_t)a.ncells_out * sizeof(unsigned short),

@@ -29,8 +29,9 @@ def _check(s, cull=False, label=""):
     return o
 
 
-# one brick of 8 x 8 x 8 cells in 293 chunks
-@pytest.mark.parametrize("n,edge", [(300_001, 0.25)])
+# one brick of 8 x 8 x 8 cells: chunk counts on both sides of the change to two
+# levels (32 chunks of 1,024 entries), and groups of 32 and 64 with a short last one
+@pytest.mark.parametrize("n,edge", [(32_768, 0.75), (32_769, 0.75), (300_001, 0.25), (1_100_000, 0.25)])
 @pytest.mark.parametrize("cull", [False, True])
 def test_one_crowded_brick_matches_oracle(n, edge, cull):
     s = _soup(n, (1, 1, 1), edge, 71, 500.0 / n)
