@@ -373,8 +373,8 @@ struct BrickArgs {
     unsigned *arrive;               // [max_slots]: chunks counted, at the brick's (or group's) first slot;
                                     // groups counted, at the brick's second
     unsigned short *counts;         // [ncells_out] objects per cell; BRICK_BIG and more: in `big`
-    uint2 *big;                     // [max_big]: cell, objects
-    unsigned max_big;
+    uint2 *big;                     // [1 << big_bits], zeroed: cell + 1, objects
+    int big_bits;
     unsigned *G;                    // the output cells array(s), ncells_out words
     long long ncells_out;
     unsigned long long *status;     // [cell_scan_tiles] look-back words, zeroed, or tile sums
@@ -397,6 +397,7 @@ constexpr unsigned BRICK_BIG = 65535u;
 unsigned brick_max_slots(unsigned count);
 unsigned brick_max_groups(unsigned count);
 unsigned brick_max_items(unsigned nbricks, unsigned count);
+int brick_big_bits(unsigned nrefs);
 unsigned long long cell_scan_tiles(long long ncells_out);
 cudaError_t launch_brick_split(const BrickArgs &a, cudaStream_t s);
 cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s);

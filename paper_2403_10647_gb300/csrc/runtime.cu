@@ -782,27 +782,27 @@ int sort_bricks(grid_ctx *c, gg::BrickArgs &a, const gg::BrickGen &bg, unsigned 
                       (unsigned *)c->keys_sorted.ptr, (unsigned *)c->vals_sorted.ptr, false, &bg));
     a.max_items = gg::brick_max_items(a.nbricks, entries);
     a.max_slots = gg::brick_max_slots(entries);
-    a.max_big = a.nrefs / gg::BRICK_BIG + 1u;
-    const size_t sizes[6] = {(size_t)a.max_items * sizeof(gg::BrickItem),
+    const size_t sizes[5] = {(size_t)a.max_items * sizeof(gg::BrickItem),
                              ((size_t)a.max_slots + gg::brick_max_groups(entries)) * gg::BRICK_CELLS * sizeof(unsigned),
                              (size_t)a.max_slots * sizeof(uint2),
                              (size_t)a.max_slots * sizeof(unsigned),
-                             (size_t)a.ncells_out * sizeof(unsigned short),
-                             (size_t)a.max_big * sizeof(uint2)};
-    size_t at[7] = {0};
-    for (int k = 0; k < 6; ++k) at[k + 1] = at[k] + ((sizes[k] + 255) & ~size_t(255));
-    GG_TRY(ensure(c, c->bricks, at[6]));
+                             (size_t)a.ncells_out * sizeof(unsigned short)};
+    size_t at[6] = {0};
+    for (int k = 0; k < 5; ++k) at[k + 1] = at[k] + ((sizes[k] + 255) & ~size_t(255));
+    GG_TRY(ensure(c, c->bricks, at[5]));
     char *base = (char *)c->bricks.ptr;
     a.items = (gg::BrickItem *)base;
     a.slots = (unsigned *)(base + at[1]);
     a.slot_meta = (uint2 *)(base + at[2]);
     a.arrive = (unsigned *)(base + at[3]);
     a.counts = (unsigned short *)(base + at[4]);
-    a.big = (uint2 *)(base + at[5]);
     const size_t tiles = (size_t)gg::cell_scan_tiles(a.ncells_out);
-    GG_TRY(ensure(c, c->k2status, tiles * 8));   // the count's look-back words are done with
+    a.big_bits = gg::brick_big_bits(a.nrefs);
+    const size_t zero = (tiles + ((size_t)1 << a.big_bits)) * 8;   // both zeroed at once
+    GG_TRY(ensure(c, c->k2status, zero));   // the count's look-back words are done with
     a.status = (unsigned long long *)c->k2status.ptr;
-    GG_CUDA(cudaMemsetAsync(a.status, 0, tiles * 8, c->stream));
+    a.big = (uint2 *)(a.status + tiles);
+    GG_CUDA(cudaMemsetAsync(a.status, 0, zero, c->stream));
     KernelScope ks(c, K_BSPLIT, 4.0 * a.nbricks);
     GG_CUDA(gg::launch_brick_split(a, c->stream));
     return GRID_OK;

@@ -60,3 +60,10 @@ def test_crowded_bricks_among_others_match_oracle():
             assert_grid_equal(g, oracle.build_grid(m.verts, m.tris, m.lam, method="counting"), f"mesh {k}")
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("cells,n,cull", [(8, 500_000, False), (8, 500_000, True), (60, 700_000, False)])
+def test_many_cells_beyond_16_bits_match_oracle(cells, n, cull):
+    s = _soup(n, (1, 1, 1), 0.7, 75, (cells - 2) / n)
+    o = _check(s, cull, str(cells))
+    assert (np.diff(o.G) >= 65_535).sum() > 4
