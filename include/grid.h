@@ -119,7 +119,8 @@ typedef struct {
                              of 2^L consecutive cells in shared memory, which also writes the
                              bucket's cell ranges.  The chain: radix passes over every key bit,
                              then range extraction (the paper's).  0 (default): with GRID_PAIRS_FUSED,
-                             bricks where they pay (from 2^21 pairs, and 4 pairs per brick entry, on):
+                             bricks where they pay (from 2^21 pairs, 4 pairs per brick entry and some 100
+                             pairs per brick on; 256 box pairs per brick in culled builds):
                              the radix passes sort one entry per 8 x 8 x 8 brick of cells and object
                              instead of its pairs, and each brick's cells and refs are written from its
                              entries; elsewhere the hybrid at up to

@@ -750,18 +750,36 @@ int brick_recs(grid_ctx *c, int64_t n, bool bricks, unsigned **bstart)
     return GRID_OK;
 }
 
-// Does it, for a scene of NO pairs in `entries` brick entries?  Where an entry
-// stands for few pairs, or there are few pairs in all, the bricks' extra steps
-// (split, count, scan: three launches) cost more than the shorter sort saves.
-// Measured, bricks against pairs: 269 against 266 us on a mesh of 1M triangles
-// with 2.4 pairs per entry, 0.42 against 1.69 ms on a soup with 57; 359 against
-// 318 us on a batch of 32,000 triangles with 1M pairs, 475 against 479 us with
-// 3.3M.
-constexpr int64_t BRICK_MIN_PAIRS = 1ll << 21, BRICK_MIN_PAIRS_PER_ENTRY = 4;
+// Does it, for NO pairs in `entries` brick entries over nbricks bricks of ncells cells?
+// Where an entry stands for few pairs, or there are few pairs in all, the bricks' extra
+// steps (split, count, scan: three launches) cost more than the shorter sort saves: 269
+// against 266 us on a mesh of 1M triangles with 2.4 pairs per entry; 359 against 318 us
+// on a batch of 32,000 triangles with 1M pairs, 475 against 479 us with 3.3M.
+//
+// A brick costs a warp of the count and a block of the fill however few entries it has
+// (about 3 ns), a sorted pair about 18 ps more than a pair placed by bricks, and a cell
+// 3 to 4 ps more in the sort's bucket steps than in the scan (9 in a batch, which
+// localizes its cells in a pass of their own): so each brick has to save so much.
+// Bricks against pairs, us, at NO + ncells / 5 (ncells / 2) of so many per brick:
+//   soups in 3D  122: 1384 / 1085, 144: 2057 / 1701, 153: 3635 / 3300, 181: 2098 / 2120, 187: 1501 / 1610
+//   flat grids    44: 1291 / 604, 76: 1375 / 926, 98: 496 / 405, 188: 1498 / 1836, 225: 278 / 289
+//   batches       81: 1192 / 784, 113: 1260 / 1093, 288: 1530 / 3051, 365: 2155 / 4221
+// (A surface that leaves most bricks empty can gain below the line too: 430 / 499 at 142.
+// How many bricks have entries is not known here.)
+//
+// Culled: the entries' masks cost 2 KB per brick with entries, so a brick has to hold more
+// box pairs: at 47 per brick 2207 / 1373, 127: 7296 / 5548, 162: 3257 / 2214, 230:
+// 4403 / 4444, 252: 320 / 330, 276: 1709 / 1826, 433: 2547 / 2835.  The masks then take at
+// most 24 bytes per box pair: the scratch stays in proportion to the pairs, as the
+// pair path's is.
+constexpr int64_t BRICK_MIN_PAIRS = 1ll << 21, BRICK_MIN_PAIRS_PER_ENTRY = 4, BRICK_MIN_PER_BRICK = 180,
+                  BRICK_MIN_PER_BRICK_CULLED = 256;
 
-bool bricks_pay(int64_t NO, int64_t entries)
+bool bricks_pay(int64_t NO, int64_t entries, int64_t nbricks, int64_t ncells, bool batch, bool cull)
 {
-    return NO >= BRICK_MIN_PAIRS && NO >= BRICK_MIN_PAIRS_PER_ENTRY * entries;
+    if (NO < BRICK_MIN_PAIRS || NO < BRICK_MIN_PAIRS_PER_ENTRY * entries) return false;
+    if (cull) return NO >= BRICK_MIN_PER_BRICK_CULLED * nbricks;
+    return NO + ncells / (batch ? 2 : 5) >= BRICK_MIN_PER_BRICK * nbricks;
 }
 
 // The first half of a brick build, after the count: entries generated and sorted
@@ -1062,7 +1080,8 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
         bg.nby = (unsigned)nby;
         bg.kb = bits_of(nbx * nby * nbz);
         bg.ob = bits_of((unsigned long long)n);
-        if (bricks_pay(NO, entries) && gg::brick_packs(bg.kb, bg.ob)) {
+        if (gg::brick_packs(bg.kb, bg.ob) &&
+            bricks_pay(NO, entries, (int64_t)(nbx * nby * nbz), I.ncells, false, c->cull)) {
             const unsigned ntiles = pair_tiles(entries);
             const bool tiles_done = ca.btile_obj && (size_t)ntiles + 1 <= ca.btile_cap &&
                                     !(c->h_ctl->err & gg::ERR_BTILE_REDO);
@@ -2072,7 +2091,7 @@ int grid_build_batched(grid_ctx *c, const grid_mesh *meshes, int32_t nmeshes, gr
     if (pairs > (uint64_t)kInt32Max) return GRID_EOVERFLOW;
     const int64_t NO = (int64_t)pairs;
     const unsigned entries = may_brick ? (unsigned)(c->h_ctl->nrefs >> gg::BRICK_SUM_BITS) : 0u;
-    const bool bricks = may_brick && NO > 0 && bricks_pay(NO, entries);
+    const bool bricks = may_brick && NO > 0 && bricks_pay(NO, entries, (int64_t)nbricks, ncells_all, true, false);
     pair_base[nm] = (unsigned)NO;
     for (int m = nm - 1; m >= 0; --m)   // an empty mesh starts where the next one does
         if (meshes[m].n == 0) pair_base[m] = pair_base[m + 1];
