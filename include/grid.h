@@ -163,9 +163,9 @@ const char *grid_version(void);
 typedef struct {
     char name[32];        /* kernel family: bounds, count_scan, tile_search, emit, upsweep_gen,
                              downsweep_gen, upsweep, downsweep, downsweep_first, downsweep_keep,
-                             extract_split, extract, bucket_split (also the bricks' items), brick_count,
-                             cell_scan, local_sort (also the bricks' refs), localize,
-                             make_pairs_per_object, cull_emit (also the bricks' culling), plan, rebase */
+                             extract_split, extract, bucket_split, local_sort, localize,
+                             make_pairs_per_object, cull_emit, plan, rebase; builds by bricks:
+                             brick_split, brick_cull, brick_count, cell_scan, brick_fill */
     int64_t launches;
     double total_ms;      /* sum of event-timed durations (0 when profiling is off) */
     double bytes;         /* sum of algorithmic bytes */

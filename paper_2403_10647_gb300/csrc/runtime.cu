@@ -60,13 +60,15 @@ struct Scratch {
 
 enum KernelId {
     K_BOUNDS, K_COUNT, K_TILES, K_EMIT, K_UP_GEN, K_DOWN_GEN, K_UP, K_DOWN, K_SPLIT, K_EXTRACT, K_LOCALIZE,
-    K_PER_OBJECT, K_CULL, K_BSPLIT, K_LOCAL, K_DOWN_ANY, K_PLAN, K_DOWN_KEEP, K_REBASE, K_BCOUNT, K_CSCAN, K_NUM
+    K_PER_OBJECT, K_CULL, K_BSPLIT, K_LOCAL, K_DOWN_ANY, K_PLAN, K_DOWN_KEEP, K_REBASE, K_BRICK_SPLIT, K_BCOUNT, K_CSCAN,
+    K_BRICK_FILL, K_BRICK_CULL, K_NUM
 };
 const char *const kKernelNames[K_NUM] = {"bounds",  "count_scan",    "tile_search",   "emit",
                                          "upsweep_gen", "downsweep_gen", "upsweep", "downsweep",
                                          "extract_split", "extract",   "localize", "make_pairs_per_object",
                                          "cull_emit", "bucket_split", "local_sort", "downsweep_first", "plan",
-                                         "downsweep_keep", "rebase", "brick_count", "cell_scan"};
+                                         "downsweep_keep", "rebase", "brick_split", "brick_count", "cell_scan",
+                                         "brick_fill", "brick_cull"};
 
 struct PendingTiming {
     int kid;
@@ -821,7 +823,7 @@ int sort_bricks(grid_ctx *c, gg::BrickArgs &a, const gg::BrickGen &bg, unsigned 
     a.status = (unsigned long long *)c->k2status.ptr;
     a.big = (uint2 *)(a.status + tiles);
     GG_CUDA(cudaMemsetAsync(a.status, 0, zero, c->stream));
-    KernelScope ks(c, K_BSPLIT, 4.0 * a.nbricks);
+    KernelScope ks(c, K_BRICK_SPLIT, 4.0 * a.nbricks);
     GG_CUDA(gg::launch_brick_split(a, c->stream));
     return GRID_OK;
 }
@@ -835,7 +837,7 @@ int fill_bricks(grid_ctx *c, const gg::BrickArgs &a, OutAlloc *out)
         GG_CUDA(gg::launch_cell_scan(a, c->stream));
     }
     if (out) GG_TRY(out->cells_ready(c, a.G, a.ncells_out));
-    KernelScope ks(c, K_LOCAL, 8.0 * a.count + 4.0 * a.ncells_out + 4.0 * a.nrefs);
+    KernelScope ks(c, K_BRICK_FILL, 8.0 * a.count + 4.0 * a.ncells_out + 4.0 * a.nrefs);
     GG_CUDA(gg::launch_brick_fill(a, c->nsm, c->stream));
     return GRID_OK;
 }
@@ -865,7 +867,7 @@ int place_bricks_culled(grid_ctx *c, gg::BrickArgs a, const gg::BrickGen &bg, un
     a.mask0 = a.word_item + a.max_words;
     GG_TRY(sort_bricks(c, a, bg, entries, nobj, tile_obj));
     {
-        KernelScope ks(c, K_CULL, 8.0 * entries + 48.0 * nobj + 4.0 * gg::BRICK_CELLS / 32 * entries);
+        KernelScope ks(c, K_BRICK_CULL, 8.0 * entries + 48.0 * nobj + 4.0 * gg::BRICK_CELLS / 32 * entries);
         GG_CUDA(gg::launch_brick_cull(a, c->nsm, c->stream));
     }
     {

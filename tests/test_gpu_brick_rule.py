@@ -61,3 +61,21 @@ def test_batches_by_bricks_where_they_pay(name):
             assert_grid_equal(g, oracle.build_grid(m.verts, m.tris, m.lam, method="counting"), f"mesh {k}")
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("cull", [False, True])
+def test_statistics_tell_brick_kernels_apart(cull):
+    import paper_2403_10647_gb300 as pg
+    pairs, bricks = {"bucket_split", "local_sort"}, {"brick_split", "brick_count", "cell_scan", "brick_fill"}
+    if cull:
+        pairs, bricks = pairs | {"cull_emit"}, bricks | {"brick_cull"}
+    c = pg.Context(0, cull=cull)
+    try:
+        for name, there, absent in (("dense", bricks, pairs), ("sparse", pairs, bricks)):
+            s = CASES[name][0]()
+            c.profile(True)
+            c.build(dev(s.verts, torch.float32), dev(s.tris, torch.int32), s.lam)
+            names = set(c.kernel_stats())
+            assert there <= names and not (absent & names), (name, names)
+    finally:
+        c.close()
