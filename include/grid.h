@@ -178,7 +178,8 @@ typedef struct {
  * shape, then the other block shape (grid_opts.tile_shape) with the best of
  * those, then the other end of the sort (grid_opts.local_bits: radix passes
  * over every key bit and range extraction if the context's setting picks
- * the hybrid for this mesh, the hybrid otherwise: local_bits -1 or -2).  Each
+ * the hybrid for this mesh, the hybrid otherwise, and if it picks bricks the one
+ * of the two that suits the mesh's pairs per cell: local_bits -1 or -2).  Each
  * candidate is timed with CUDA events on the context's stream: the median of
  * `reps` builds after one warm-up (reps <= 0 means 3).  Every candidate gives
  * the same grid, so tuning changes speed only.  *chosen (may be NULL) gets

@@ -93,6 +93,7 @@ struct grid_ctx {
     int local_bits = 0;          // grid_opts.local_bits
     int64_t fallbacks = 0;       // hybrid placements redone by radix passes over every key bit
     int64_t plan_redos = 0;      // builds whose device M differed from the host's
+    bool by_bricks = false;      // the last build placed its pairs by bricks
 
     Ctl *d_ctl = nullptr;        // device control block: one of the two ctls
     Ctl *ctls[2] = {nullptr, nullptr};
@@ -570,6 +571,15 @@ bool use_hybrid(const grid_ctx *c, int64_t count, int64_t ncells)
     return (double)count <= LOCAL_PAIRS_PER_CELL * (double)std::max<int64_t>(ncells, 1);
 }
 
+// The local_bits that an autotuner compares with the context's own choice, which its
+// last build (of count pairs) took: what builds by sorted pairs use at this
+// density if that was bricks, else radix passes over every key bit if it was the
+// hybrid, and the hybrid if it was not.
+int other_sort_end(const grid_ctx *c, int64_t count, int64_t ncells)
+{
+    return use_hybrid(c, count, ncells) == c->by_bricks ? -2 : -1;
+}
+
 // Local bits L of the hybrid placement for `count` pairs over `ncells` cells
 // with key_bits-bit keys: the radix passes sort the bits from L up and one
 // block per bucket of 2^L cells sorts the rest.  L_hi is the largest L whose
@@ -961,6 +971,7 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
     if (n > 0 && (!verts || !tris)) return GRID_EINVAL;
     grid_info I;
     unsigned *cells = nullptr, *refs = nullptr;
+    c->by_bricks = false;
     if (n == 0) {
         const float z[3] = {0.f, 0.f, 0.f};
         GG_TRY(plan(z, z, 0, lambda, &I));
@@ -1084,6 +1095,7 @@ int build_core(grid_ctx *c, const float *verts, int64_t nverts, const int32_t *t
         bg.ob = bits_of((unsigned long long)n);
         if (gg::brick_packs(bg.kb, bg.ob) &&
             bricks_pay(NO, entries, (int64_t)(nbx * nby * nbz), I.ncells, false, c->cull)) {
+            c->by_bricks = true;
             const unsigned ntiles = pair_tiles(entries);
             const bool tiles_done = ca.btile_obj && (size_t)ntiles + 1 <= ca.btile_cap &&
                                     !(c->h_ctl->err & gg::ERR_BTILE_REDO);
@@ -1628,15 +1640,11 @@ int grid_ctx_autotune(grid_ctx *c, const float *verts, int64_t nverts, const int
             }
         }
     }
-    // then the other way to finish the sort and the range steps: radix
-    // passes over every key bit and extraction when the context uses the
-    // per-bucket counting sort, and the automatic hybrid otherwise
+    // then the other way to finish the sort and the range steps (other_sort_end)
     int best_lb = saved_lb;
     if (rc == GRID_OK) {
         c->shape = best_shape;
-        // the context's own choice for this mesh (its pair and cell counts
-        // come from one more build), then the other one: radix passes over
-        // every key bit if it chose the hybrid, the hybrid if it did not
+        // the context's own choice for this mesh comes from one more build
         grid_info probe{};
         grid_buf cells{}, refs{};
         PoolOut po(&cells, &refs);
@@ -1644,7 +1652,7 @@ int grid_ctx_autotune(grid_ctx *c, const float *verts, int64_t nverts, const int
         rc = build_core(c, verts, nverts, tris, n, lambda, &probe, po);
         grid_buf_free(c, &cells);
         grid_buf_free(c, &refs);
-        c->local_bits = use_hybrid(c, probe.nrefs, probe.ncells) ? -1 : -2;
+        c->local_bits = other_sort_end(c, probe.nrefs, probe.ncells);
         double med = 0.0;
         if (rc == GRID_OK) rc = time_setting(&med);
         if (rc == GRID_OK) {
@@ -1756,7 +1764,7 @@ int grid_ctx_autotune_batched(grid_ctx *c, const grid_mesh *meshes, int32_t nmes
         }
         grid_buf_free(c, &probe_cells);
         grid_buf_free(c, &probe_refs);
-        c->local_bits = use_hybrid(c, np, nc) ? -1 : -2;
+        c->local_bits = other_sort_end(c, np, nc);
         double med = 0.0;
         if (rc == GRID_OK) rc = time_setting(&med);
         if (rc == GRID_OK) {
@@ -2094,6 +2102,7 @@ int grid_build_batched(grid_ctx *c, const grid_mesh *meshes, int32_t nmeshes, gr
     const int64_t NO = (int64_t)pairs;
     const unsigned entries = may_brick ? (unsigned)(c->h_ctl->nrefs >> gg::BRICK_SUM_BITS) : 0u;
     const bool bricks = may_brick && NO > 0 && bricks_pay(NO, entries, (int64_t)nbricks, ncells_all, true, false);
+    c->by_bricks = bricks;
     pair_base[nm] = (unsigned)NO;
     for (int m = nm - 1; m >= 0; --m)   // an empty mesh starts where the next one does
         if (meshes[m].n == 0) pair_base[m] = pair_base[m + 1];
