@@ -1296,9 +1296,10 @@ struct ScratchOut : OutAlloc {
     }
 };
 
-// Outputs in the context's scratch, bound for host buffers: once the refs
-// are final their device-to-host copy starts on the context's copy stream,
-// so it overlaps range extraction on the build stream.
+// Outputs in the context's scratch, bound for host buffers: once the refs (in a
+// brick build the cells) are final their device-to-host copy starts on the
+// context's copy stream, so it overlaps range extraction (the fill of the refs)
+// on the build stream.
 struct HostOut : ScratchOut {
     int32_t *h_cells, *h_refs;   // both or neither
     int64_t cells_cap, refs_cap;
@@ -1307,15 +1308,17 @@ struct HostOut : ScratchOut {
         : h_cells(hc && hr ? hc : nullptr), h_refs(hc && hr ? hr : nullptr), cells_cap(ccap), refs_cap(rcap)
     {
     }
+    // both buffers hold the grid (the sizes are those of alloc): else GRID_ENOSPC, and nothing is written
+    bool fits() const { return h_cells && ncells1 <= cells_cap && nrefs <= refs_cap; }
     // a brick build's cells are final while its refs are still being written
     int cells_ready(grid_ctx *c, const unsigned *cells, int64_t count) override
     {
-        if (!h_cells || count > cells_cap) return GRID_OK;
+        if (!fits()) return GRID_OK;
         return copy_out(c, h_cells, cells, count, &cells_copied);
     }
     int refs_ready(grid_ctx *c, const unsigned *refs, int64_t count) override
     {
-        if (!h_refs || count <= 0 || count > refs_cap) return GRID_OK;   // copied after the build, or ENOSPC
+        if (!fits() || count <= 0) return GRID_OK;
         return copy_out(c, h_refs, refs, count, &copied);
     }
     static int copy_out(grid_ctx *c, int32_t *dst, const unsigned *src, int64_t count, bool *copied)
@@ -1824,7 +1827,7 @@ int grid_build_host(grid_ctx *c, const float *h_verts, int64_t nverts, const int
         GG_TRY(build_core(c, (const float *)c->in_verts.ptr, nverts, (const int32_t *)c->in_tris.ptr, n, lambda,
                           &I, so));
         if (info) *info = I;
-        if (!h_cells || !h_refs || cells_cap < so.ncells1 || refs_cap < so.nrefs) return GRID_ENOSPC;
+        if (!so.fits()) return GRID_ENOSPC;
         if (!so.cells_copied)
             GG_CUDA(cudaMemcpyAsync(h_cells, c->out_cells.ptr, (size_t)so.ncells1 * 4, cudaMemcpyDeviceToHost,
                                     c->stream));
