@@ -509,12 +509,19 @@ __global__ void __launch_bounds__(32 * COUNT_WARPS, 8) brick_count_kernel(BrickA
 // and the test runs over the list, a pair per lane.
 //
 // That bound, T: the test drops a cell when the three projections p_k = n . w_k
-// all lie beyond R = S (1/2 + max|w| 2^-16 + 2^-10) on one side.  With n
-// the FP32 cross product of FP32 edges of length at most L per component, n . e
-// is not zero but below 16 u L^3 (u = 2^-24), and the rounding of a projection
-// below 4 u S W <= 24 u L^2 W for W >= max|w| over the brick; the plane's own
-// value here is off by no more.  T = S (1/2 + W 2^-16 + 2^-10) (1 + 2^-10) +
-// 2^-18 L^2 (L + W) exceeds R by the sum of these.
+// all lie beyond R = S (1/2 + max|w| 2^-16 + 2^-10) on one side, S = |n_x| + |n_y| +
+// |n_z|.  The cell is dropped here when its plane value v, p_0 but for rounding,
+// lies beyond T: so T has to exceed R by what the three can differ from v.  Let
+// the FP32 edges have components up to L, and |w| be up to W over the
+// brick; S <= 4 L^2 (a 3 x 3 determinant of entries up to 1 is at most 4).
+//  - n . (q_k - q_0) is not zero: each component of the FP32 cross product is off by
+//    4 u L^2 (u = 2^-24) and each edge by u L, which makes 16 u L^3 for k = 1 and 28 u
+//    L^3 for k = 2 (the three rounded edges do not add up to zero).
+//  - The test's rounding of a projection (w, three products, two sums): 4 u S W.
+//  - The rounding of v (q - c0, three fused steps to the brick's first cell, three
+//    to this one): 7 u S W.
+// Together 28 u L^3 + 11 u S W <= 28 u L^3 + 44 u L^2 W.  T = S (1/2 + W 2^-16 + 2^-10)
+// (1 + 2^-10) + 2^-18 L^2 (L + W) exceeds R by more than 64 u L^3 + 64 u L^2 W.
 //
 // Bound by issue (73% of cycles).  Tests and compaction pair by pair, ahead of a
 // sort of the pairs, then this kernel: 1150 -> 297 us on the soup of 1M triangles,
