@@ -28,20 +28,28 @@ constexpr unsigned SPIN_LIMIT = 1u << 20;
 constexpr int MAX_PASSES = 4;
 constexpr int MAX_RADIX = 1 << 11;
 
-// Per-build control block, zeroed by one memset before the first kernel.
+// Per-build control block, zero before the first kernel: a context has two, and
+// a single-mesh build's bounds kernel zeroes the one for the next build; where no
+// build did, a memset does.  A count that is run again (the host's grid
+// metadata in place of the device's) starts from err, tickets[0], npairs and count_done
+// zeroed anew; it writes nrefs over.
 struct Ctl {
     unsigned lo_inv[3];         // atomicMax of ~ordered(min coordinate) per axis
     unsigned hi_ord[3];         // atomicMax of ordered(max coordinate) per axis
     unsigned err;               // ERR_* bits
-    unsigned bounds_done;       // blocks that finished: bounds, count/scan, the build's last kernel
+    unsigned bounds_done;       // blocks of the bounds kernel that finished (the last one plans)
     unsigned long long nrefs;   // NO, written by the last count/scan tile (with the brick entries in the
                                 // bits from BRICK_SUM_BITS on when it counted them)
-    unsigned tickets[8];        // tile tickets: [0] count/scan, [5] cell scan, [7] culling emit; counts: [1] cells of many objects,
-                                // [2] the hybrid placement's bucket groups, [3] the brick items,
-                                // [4] their chunk slots, [6] the empty bricks
-    unsigned long long nkept;   // pairs the culling emit kept, written by its last tile
+    unsigned tickets[8];        // tile tickets: [0] count/scan, [5] cell scan (its look-back's tiles, or the
+                                // blocks of its first pass that finished), [7] culling emit; counts: [1] cells
+                                // of many objects, [2] the hybrid placement's bucket groups or a culled brick
+                                // build's words of entries, [3] the brick items, [4] their chunk slots, [6] the
+                                // empty bricks
+    unsigned long long nkept;   // pairs that culling kept: by the culling emit's last tile, or added up by the
+                                // brick count
     unsigned long long npairs;  // a count with brick entries: NO added up on its own, exact
-    unsigned count_done, place_done;
+    unsigned count_done, place_done;   // blocks of count/scan, and of the placement's last kernel, that
+                                       // finished (publish_ctl)
     // grid metadata M computed on the device from the bounds above (plan_kernel),
     // for count/scan to read without a host round trip; the host checks it
     // against its own plan from the same bounds
