@@ -315,22 +315,35 @@ def _bench_batched_timed(ctx, meshes, args, reps):
 
 
 def bench_pair_gen(scene, reps: int = 5):
-    """Pair-generation ablation on one scene: the default (pairs generated by
-    the first sort pass's counting kernel and stored once), the first pass
-    regenerating them in both of its kernels, the paper's unfused chain (a
-    kernel of its own writes them, then the sort) and the sorted grid's
-    one-thread-per-object MakePairs, each timed per build with CUDA events
-    and per kernel with the library's own event accounting."""
+    """Pair-generation ablation on one scene, by sorted pairs throughout: pairs
+    generated by the first sort pass's counting kernel and stored once, the
+    first pass regenerating them in both of its kernels, the paper's unfused
+    chain (a kernel of its own writes them, then the sort) and the sorted
+    grid's one-thread-per-object MakePairs, each timed per build with CUDA
+    events and per kernel with the library's own event accounting; and, where
+    the default builds by bricks, that build (its first sort pass generates
+    brick entries)."""
     import torch
     import paper_2403_10647_gb300 as pg
     v = torch.from_numpy(scene.verts).cuda()
     t = torch.from_numpy(scene.tris).cuda()
     out = {"n_tris": scene.n}
     ref = None
-    for mode in ("fused", "regen", "emit", "per_object"):
-        c = pg.Context(0, pair_gen=mode)
+    local_bits = 0   # what sorted pairs end in at this density, for the fused mode (the others never take bricks)
+    for mode in ("default", "fused", "regen", "emit", "per_object"):
+        if mode == "default":
+            c = pg.Context(0)
+        else:
+            c = pg.Context(0, pair_gen=mode, local_bits=local_bits if mode == "fused" else 0)
         try:
+            c.profile(True)
             g = c.build(v, t, scene.lam)
+            if mode == "default":
+                local_bits = -1 if c.sort_plan(g.info.key_bits, g.info.nrefs, g.info.ncells)[0] == -1 else -2
+                if "brick_fill" not in c.kernel_stats():
+                    continue   # the default is the fused mode
+                mode = "bricks"
+            c.profile(False)
             if ref is None:
                 ref = g
                 out["nrefs"] = g.info.nrefs
@@ -351,7 +364,7 @@ def bench_pair_gen(scene, reps: int = 5):
             st = c.kernel_stats()
             c.profile(False)
             gen = {"fused": ("upsweep_gen",), "regen": ("upsweep_gen", "downsweep_gen"),
-                   "emit": ("tile_search", "emit"), "per_object": ("make_pairs_per_object",)}[mode]
+                   "emit": ("tile_search", "emit"), "per_object": ("make_pairs_per_object",), "bricks": ("upsweep_gen",)}[mode]
             out[mode] = {"ms_per_build": e0.elapsed_time(e1) / reps,
                          "pair_generation_ms": sum(st[k]["ms"] for k in gen if k in st) / reps,
                          "pair_generation_kernels": list(gen)}
@@ -729,6 +742,12 @@ def run_ours(args, rank, world, local):
     lbits, rpasses = ctx.sort_plan(info.key_bits, nrefs, info.ncells)
     high_bits = info.key_bits - max(lbits, 0)
     digit = max(8, -(-high_bits // rpasses)) if rpasses else 8
+    plan = {"placement": "chain" if lbits == -1 else "hybrid", "local_bits": lbits, "radix_passes": rpasses,
+            "radix_digit_bits": digit}
+    if "brick_fill" in stats:   # the passes sort brick entries: ncells is not what they see
+        digit = 8
+        plan = {"placement": "bricks", "radix_passes": round(stats["upsweep"]["launches"] / args.steps) + 1
+                if "upsweep" in stats else 1}
     traffic = traffic_from_profiles(dom, digit, nrefs)
     roof = {"bound": "hbm", "kernel": dom, "achieved": kern[dom]["gbs"], "peak": peak, "unit": "GB/s",
             "frac": kern[dom]["gbs"] / peak, "traffic": traffic, "peak_kind": peak_kind,
@@ -790,7 +809,7 @@ def run_ours(args, rank, world, local):
         "config": {"workload": args.workload, "n_tris": scene.n, "lambda": scene.lam, "grid": list(info.res),
                    "ncells": info.ncells, "nrefs": nrefs, "key_bits": info.key_bits,
                    "radix_bits": args.radix_bits,
-                   "sort_plan": {"local_bits": lbits, "radix_passes": rpasses, "radix_digit_bits": digit},
+                   "sort_plan": plan,
                    "pair_gen": args.pair_gen or "fused", "cull": bool(args.cull), "tile_shape": args.tile_shape,
                    "autotune_choice": (f"{tuned['radix_bits']}/{tuned['pair_gen']}/{tuned['tile_shape']}"
                                        if tuned else None),
