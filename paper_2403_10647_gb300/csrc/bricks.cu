@@ -1418,10 +1418,12 @@ cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Beyond 4 pairs per cell the larger stage wins, below the more resident blocks:
-// 132 against 150 us on the soup of 1M triangles (19 pairs per cell), 812
-// against 724 us on the building of 10M (2.4; an earlier form of the kernel).
-constexpr double DENSE_PAIRS_PER_CELL = 4.0;
+// In crowded cells the larger stage wins, in the others the more resident blocks.
+// Larger against smaller, us, at so many pairs per cell: buildings 2.5: 186 / 147,
+// 4.5: 101 / 99, 6.3: 91 / 97; soups of 4M triangles 4.0: 242 / 199, 6.8: 305 / 283, 7.9:
+// 206 / 251, 13.6: 268 / 349, 128: 559 / 604; of 400,000 4.0: 31 / 29, 6.8: 38 / 46; soups of
+// uneven triangles 19.5: 134 / 203.
+constexpr double DENSE_PAIRS_PER_CELL = 6.0;
 
 cudaError_t launch_brick_fill(const BrickArgs &a, int nsm, cudaStream_t s)
 {
