@@ -1155,15 +1155,6 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
         unsigned dst[4], num[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) dst[k] = num[k] = 0u;
-        // a chunk's rows: the brick's chunks before it come first in each cell
-        const unsigned *before = nullptr, *before_group = nullptr;
-        if (it.slot != NO_SLOT) {
-            const uint2 meta = a.slot_meta[it.slot];
-            before = a.slots + (size_t)it.slot * BRICK_CELLS + c0;
-            if (meta.y > MERGE_CHUNKS)
-                before_group = a.slots + c0 +
-                               (size_t)(group_row(a, meta.x) + (it.slot - meta.x) / merge_group(meta.y)) * BRICK_CELLS;
-        }
         if (y < d.ny && z < d.nz) {
             const unsigned *gp = a.G + it.cell0 + x + it.rx * y + it.rxy * z;
             unsigned g[5];
@@ -1175,10 +1166,18 @@ __global__ void __launch_bounds__(32 * FILL_WARPS, MIN_BLOCKS) brick_fill_kernel
                     dst[k] = it.base + g[k];
                     num[k] = g[k + 1] - g[k];
                     bad |= num[k] > a.nrefs || dst[k] > a.nrefs - num[k];
-                    // this chunk's share of the cell is counted below
-                    if (before) dst[k] += __ldg(before + k);
-                    if (before_group) dst[k] += __ldg(before_group + k);
+                    // the cell's other chunks come first; this one's share is counted below
+                    if (it.slot != NO_SLOT) dst[k] += __ldg(a.slots + (size_t)it.slot * BRICK_CELLS + c0 + k);
                 }
+            }
+        }
+        if (it.slot != NO_SLOT) {   // those of a brick in many chunks: the groups before this one's
+            const uint2 meta = a.slot_meta[it.slot];
+            if (meta.y > MERGE_CHUNKS && y < d.ny && z < d.nz) {
+                const unsigned row = group_row(a, meta.x) + (it.slot - meta.x) / merge_group(meta.y);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (x + k < d.nx) dst[k] += __ldg(a.slots + (size_t)row * BRICK_CELLS + c0 + k);
             }
         }
         __syncthreads();   // the previous item's masks and objects are read
