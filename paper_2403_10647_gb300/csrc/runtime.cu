@@ -779,6 +779,17 @@ int brick_recs(grid_ctx *c, int64_t n, bool bricks, unsigned **bstart)
 // (A surface that leaves most bricks empty can gain below the line too: 430 / 499 at 142.
 // How many bricks have entries is not known here.)
 //
+// Grids of few cells sort their pairs in one or two passes, of 6 and 10 ps a pair; an
+// entry costs 36 to 47 ps there and the bricks' extra launches 25 to 50 us.  So one pass of
+// 8-bit digits (256 cells) asks for NO >= 8 entries + 2^23, one of 9 bits for 6 entries +
+// 2^22, two passes for 4 entries + 2^21.  Bricks against pairs, us, at NO (entries) in millions:
+//   64 cells    4.0 (0.5): 192 / 137, 10.7 (0.5): 189 / 195, 18.7 (1.5): 293 / 307, 50 (4): 517 / 608
+//   343 cells   5.1 (0.5): 184 / 170, 9.8 (1.5): 278 / 258, 26 (4): 521 / 512, 41 (4): 545 / 665
+//   4,096       2.7 (0.6): 178 / 155, 4.0 (0.6): 180 / 181, 8.0 (1.7): 267 / 262, 21 (4.6): 489 / 514
+// Bricks of a line along y or z hold 8 cells: 640 / 435 at 4.1 pairs per entry, 1178 / 984
+// culled, so such bricks ask for 6.  Other culled builds gain in few cells too (855 / 922
+// at 8 cells, 991 / 1206 at 64): there the pairs are tested in memory first.
+//
 // Culled: the entries' masks cost 2 KB per brick with entries, so a brick has to hold more
 // box pairs: at 47 per brick 2207 / 1373, 127: 7296 / 5548, 162: 3257 / 2214, 230:
 // 4403 / 4444, 252: 320 / 330, 276: 1709 / 1826, 433: 2547 / 2835.  The masks then take at
@@ -790,7 +801,12 @@ constexpr int64_t BRICK_MIN_PAIRS = 1ll << 21, BRICK_MIN_PAIRS_PER_ENTRY = 4, BR
 bool bricks_pay(int64_t NO, int64_t entries, int64_t nbricks, int64_t ncells, bool batch, bool cull)
 {
     if (NO < BRICK_MIN_PAIRS || NO < BRICK_MIN_PAIRS_PER_ENTRY * entries) return false;
+    if (!batch && ncells < 16 * nbricks && NO < 6 * entries) return false;
     if (cull) return NO >= BRICK_MIN_PER_BRICK_CULLED * nbricks;
+    if (!batch && ncells <= 1 << 16) {
+        const int k = ncells <= 1 << 8 ? 2 : ncells <= 1 << 9 ? 1 : 0;
+        if (NO < (4 + 2 * k) * entries + (BRICK_MIN_PAIRS << k)) return false;
+    }
     return NO + ncells / (batch ? 2 : 5) >= BRICK_MIN_PER_BRICK * nbricks;
 }
 

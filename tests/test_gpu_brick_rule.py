@@ -28,6 +28,16 @@ CASES = {
     "sparse": (lambda: _scene(70_000, 4.5, 512.0), False, False),             # 60
     "flat_dense": (lambda: _scene(60_000, 12, 8.0, flat=True), True, True),   # 1,270
     "flat_sparse": (lambda: _scene(240_000, 4, 64.0, flat=True), False, False),   # 27
+    # few cells, sorted in one or two passes: enough pairs beyond so many per entry
+    "18_cells": (lambda: _scene(600_000, 1, 8 / 600_000), False, True),
+    "64_cells_few": (lambda: _scene(500_000, 1, 62 / 500_000), False, True),
+    "64_cells": (lambda: _scene(700_000, 3, 62 / 700_000), True, True),
+    "343_cells_few": (lambda: _scene(500_000, 1, 340 / 500_000), False, True),
+    "343_cells": (lambda: _scene(500_000, 3, 340 / 500_000), True, True),
+    "4096_cells_few": (lambda: _scene(600_000, 1.1, 4_090 / 600_000), False, True),
+    "4096_cells": (lambda: _scene(600_000, 3, 4_090 / 600_000), True, True),
+    "line_z_few": (lambda: _soup(600_000, (0, 0, 1), 0.012, 82, 1_000 / 600_000), False, False),
+    "line_z": (lambda: _soup(200_000, (0, 0, 1), 0.1, 82, 1_000 / 200_000), True, True),
 }
 
 
