@@ -1402,6 +1402,8 @@ cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s)
     return cudaGetLastError();
 }
 
+int cell_scan_launches(long long ncells_out) { return ncells_out > SCAN_ONE_PASS ? 2 : 1; }
+
 cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s)
 {
     const unsigned tiles = (unsigned)cell_scan_tiles(a.ncells_out);

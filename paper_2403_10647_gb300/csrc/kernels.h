@@ -399,6 +399,7 @@ unsigned brick_max_groups(unsigned count);
 unsigned brick_max_items(unsigned nbricks, unsigned count);
 int brick_big_bits(unsigned nrefs);
 unsigned long long cell_scan_tiles(long long ncells_out);
+int cell_scan_launches(long long ncells_out);   // kernels of launch_cell_scan
 cudaError_t launch_brick_split(const BrickArgs &a, cudaStream_t s);
 cudaError_t launch_brick_count(const BrickArgs &a, int nsm, cudaStream_t s);
 cudaError_t launch_cell_scan(const BrickArgs &a, cudaStream_t s);

@@ -228,15 +228,15 @@ cudaEvent_t take_event(grid_ctx *c)
     return e;
 }
 
-// Brackets one kernel launch: counts it, adds its algorithmic bytes and, when
-// profiling, records events on the launching stream around it.
+// Brackets one kernel launch (or n of one family): counts it, adds its algorithmic
+// bytes and, when profiling, records events on the launching stream around it.
 struct KernelScope {
     grid_ctx *c;
     int kid;
     cudaEvent_t start = nullptr;
-    KernelScope(grid_ctx *ctx, int k, double bytes) : c(ctx), kid(k)
+    KernelScope(grid_ctx *ctx, int k, double bytes, int n = 1) : c(ctx), kid(k)
     {
-        c->launches[kid] += 1;
+        c->launches[kid] += n;
         c->kernel_bytes[kid] += bytes;
         if (c->profile) {
             start = take_event(c);
@@ -859,7 +859,7 @@ int sort_bricks(grid_ctx *c, gg::BrickArgs &a, const gg::BrickGen &bg, unsigned 
 int fill_bricks(grid_ctx *c, const gg::BrickArgs &a, OutAlloc *out)
 {
     {
-        KernelScope ks(c, K_CSCAN, 6.0 * a.ncells_out);
+        KernelScope ks(c, K_CSCAN, 6.0 * a.ncells_out, gg::cell_scan_launches(a.ncells_out));
         GG_CUDA(gg::launch_cell_scan(a, c->stream));
     }
     if (out) GG_TRY(out->cells_ready(c, a.G, a.ncells_out));

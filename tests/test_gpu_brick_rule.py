@@ -89,3 +89,16 @@ def test_statistics_tell_brick_kernels_apart(cull):
             assert there <= names and not (absent & names), (name, names)
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("name,launches", [("dense", 1), ("near", 2)])   # 0.5M and 8M cells: one pass, two
+def test_scan_launches_are_counted(name, launches):
+    import paper_2403_10647_gb300 as pg
+    s = CASES[name][0]()
+    c = pg.Context(0)
+    try:
+        c.profile(True)
+        c.build(dev(s.verts, torch.float32), dev(s.tris, torch.int32), s.lam)
+        assert c.kernel_stats()["cell_scan"]["launches"] == launches
+    finally:
+        c.close()
