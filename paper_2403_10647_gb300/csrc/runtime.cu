@@ -787,8 +787,8 @@ int brick_recs(grid_ctx *c, int64_t n, bool bricks, unsigned **bstart)
 //   343 cells   5.1 (0.5): 184 / 170, 9.8 (1.5): 278 / 258, 26 (4): 521 / 512, 41 (4): 545 / 665
 //   4,096       2.7 (0.6): 178 / 155, 4.0 (0.6): 180 / 181, 8.0 (1.7): 267 / 262, 21 (4.6): 489 / 514
 // Bricks of a line along y or z hold 8 cells: 640 / 435 at 4.1 pairs per entry, 1178 / 984
-// culled, so such bricks ask for 6.  Other culled builds gain in few cells too (855 / 922
-// at 8 cells, 991 / 1206 at 64): there the pairs are tested in memory first.
+// culled, so such bricks ask for 6.  Other culled builds gain in few cells too (991 / 1206
+// at 64 cells): there the pairs are tested in memory first.
 //
 // Culled: the entries' masks cost 2 KB per brick with entries, so a brick has to hold more
 // box pairs: at 47 per brick 2207 / 1373, 127: 7296 / 5548, 162: 3257 / 2214, 230:
